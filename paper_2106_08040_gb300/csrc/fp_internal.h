@@ -75,6 +75,10 @@ struct FpRadau {
     double gam;                      // real eigenvalue of a^{-1}
     double alp[3], bet[3];           // complex pairs alp +- i bet (bet > 0)
     double e[FP_SMAX], g0;           // err_pre = h g0 f(t_n, y_n) + sum_i e_i Z_i
+    // the constants of the FP32 transformations, rounded once on the host: a
+    // conversion in the kernel would take an FP64-pipe slot per use
+    float Tf[FP_SMAX][FP_SMAX], Tif[FP_SMAX][FP_SMAX], Kf[FP_SMAX][FP_SMAX];
+    float gamf, alpf[3], betf[3];
 };
 
 // Host-built tables (device copies live in the context).

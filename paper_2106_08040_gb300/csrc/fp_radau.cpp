@@ -212,5 +212,13 @@ int fp_build_radau(int s, FpRadau* r) {
         for (int i = 0; i < s; ++i) e += (bh[i] - a[(s - 1) * s + i]) * ai[i * s + j];
         r->e[j] = e;
     }
+    for (int i = 0; i < s; ++i)
+        for (int j = 0; j < s; ++j) {
+            r->Tf[i][j] = (float)r->T[i][j];
+            r->Tif[i][j] = (float)r->Ti[i][j];
+            r->Kf[i][j] = (float)r->K[i][j];
+        }
+    r->gamf = (float)r->gam;
+    for (int q = 0; q < 3; ++q) { r->alpf[q] = (float)r->alp[q]; r->betf[q] = (float)r->bet[q]; }
     return FP_OK;
 }

@@ -285,6 +285,54 @@ __device__ void apply_A(const double* __restrict__ x, double* __restrict__ y, co
     for (int i = threadIdx.x; i < N; i += NT) y[i] = apply_row(i, x, sc, diag, N, T);
 }
 
+// out_j = A_j x_j for the S stage states x [S][N] with the scalars sc[j].  The
+// FP64 pipe bounds it (24 operations a row at 2 a clock and SM); a thread takes
+// one row for all stages, so a coupling's coefficient and source index are
+// fetched once and S independent chains hide each other's latency.  The rows
+// beyond the last multiple of NT go one (row, stage) pair to a thread: a second
+// pass of whole rows would leave most warps idle behind it.
+template <int S>
+__device__ __forceinline__ void apply_stages(const double* __restrict__ x, double* __restrict__ out, const AScal* sc,
+                                             const double* __restrict__ diag, int N, const DevTab& T) {
+    const int nfull = N - N % NT;
+    for (int i = threadIdx.x; i < nfull; i += NT) {
+        const double* cf = T.coef4 + i;
+        const int* sr = T.src + i;
+        const int ld = T.nrow;
+        double g[S][4];
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) g[s][q] = 0.0;
+#pragma unroll
+        for (int k = 0; k < FP_NSLOT; ++k) {
+            const int j = __ldg(sr + k * ld);
+            const double c = __ldg(cf + k * ld);
+            const bool in = (unsigned)j < (unsigned)N;
+#pragma unroll
+            for (int s = 0; s < S; ++s) {
+                const double v = in ? x[s * N + j] : 0.0;
+                g[s][grp4_of(k)] = fma(c, v, g[s][grp4_of(k)]);
+            }
+        }
+        const double dg = diag[i];
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+            double acc = dg * x[s * N + i];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc = fma(sc[s].s4[q], g[s][q], acc);
+            out[s * N + i] = acc;
+        }
+    }
+    const int nrest = N - nfull;
+    if (nrest == 0) return;
+    int s = 0, i = threadIdx.x;
+    for (int e = threadIdx.x; e < S * nrest; e += NT, i += NT) {
+        while (i >= nrest) { i -= nrest; ++s; }
+        out[s * N + nfull + i] = apply_row(nfull + i, x + s * N, sc[s], diag, N, T);
+    }
+}
+
 // ------------------------------------------------------- per-CTA state ----
 template <int S>
 struct Ctx {
@@ -492,11 +540,11 @@ __device__ void factorize(Ctx<S>& C, const AScal& sc, double h, int* pp, float2*
     const size_t nm2 = (size_t)C.ly.nmax * C.ly.nmax;
     for (int mu = 0; mu <= L; ++mu) {
         if (sys == 0) {
-            group_factor_block<float, S, GW, RS>(C, mu, (float)RAD<S>().gam, gs, (float)h, C.Xr, C.fr + C.foff[mu],
+            group_factor_block<float, S, GW, RS>(C, mu, RAD<S>().gamf, gs, (float)h, C.Xr, C.fr + C.foff[mu],
                                                  pp, (float*)colbuf, gw, 1);
         } else if (sys <= NC) {
             const int q = sys - 1;
-            const float2 shift = make_float2((float)RAD<S>().alp[q], -(float)RAD<S>().bet[q]);
+            const float2 shift = make_float2(RAD<S>().alpf[q], -RAD<S>().betf[q]);
             group_factor_block<float2, S, GW, RS>(C, mu, shift, gs, (float)h, C.Xc + q * nm2,
                                                   C.fc + (size_t)q * C.ly.fsum + C.foff[mu], pp + FP_PP_SYS * sys,
                                                   colbuf + FP_CB_SYS * sys, gw, 1 + sys);
@@ -774,14 +822,12 @@ __device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, dou
     NewtonResult res{false, false, 0.f, 0.f, 0};
     float prev = 3.0e38f;
     eta = powf(fmaxf(eta, 1e-7f), 0.8f);
+    for (int j = 0; j < S; ++j)
+        for (int i = threadIdx.x; i < N; i += NT) C.yb[j * N + i] = C.y[i] + C.Z[j * N + i];
+    __syncthreads();
     for (int it = 0; it < maxit; ++it) {
         // F_j = A(t + c_j h)(y + Z_j) for all stages in one pass, FP64
-        for (int e = threadIdx.x; e < S * N; e += NT) C.yb[e] = C.y[e % N] + C.Z[e];
-        __syncthreads();
-        for (int e = threadIdx.x; e < S * N; e += NT) {
-            const int j = e / N, i = e - j * N;
-            C.F[e] = apply_row(i, C.yb + j * N, sh.scj[j], C.diag, N, T);
-        }
+        apply_stages<S>(C.yb, C.F, sh.scj, C.diag, N, T);
         __syncthreads();
         // residual R = -Z + h a F (FP64) -> right-hand sides K R (FP32, block order)
         for (int b = threadIdx.x; b < N; b += NT) {
@@ -802,7 +848,7 @@ __device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, dou
             for (int k = 0; k < S; ++k) {
                 float acc = 0.f;
 #pragma unroll
-                for (int j = 0; j < S; ++j) acc = fmaf((float)RAD<S>().K[k][j], Rk[j], acc);
+                for (int j = 0; j < S; ++j) acc = fmaf(RAD<S>().Kf[k][j], Rk[j], acc);
                 q[k] = acc;
             }
             C.rr[b] = q[0];
@@ -835,12 +881,14 @@ __device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, dou
             for (int k = 0; k < S; ++k) {
                 float dz = 0.f;
 #pragma unroll
-                for (int j = 0; j < S; ++j) dz = fmaf((float)RAD<S>().T[k][j], dW[j], dz);
-                C.Z[k * N + i] += (double)dz;
+                for (int j = 0; j < S; ++j) dz = fmaf(RAD<S>().Tf[k][j], dW[j], dz);
+                const double zn = C.Z[k * N + i] + (double)dz;
+                C.Z[k * N + i] = zn;
+                C.yb[k * N + i] = C.y[i] + zn;                 // the next iteration's stage states
                 dm = nanmax(dm, fabsf(dz));
             }
         }
-        const float dmax = block_max(dm, sh.red);
+        const float dmax = block_max(dm, sh.red);              // (its barriers order yb before the next apply)
         ++res.iters;
         res.dmax = dmax;
         if (!(dmax <= 3.0e38f)) { res.nonfinite = true; break; }
@@ -1338,16 +1386,16 @@ __device__ int adjoint_stages(Ctx<S>& C, const DevTab& T, double hs, double h_f,
     int nflat = 0;
     for (int it = 0; it < maxit; ++it) {
         // v_i = sum_j a_ji zeta_j ; w_i = A_i^T v_i
-        for (int e = threadIdx.x; e < S * N; e += NT) {
-            const int i = e / N, r = e - i * N;
+        for (int e = threadIdx.x, i = 0, r = threadIdx.x; e < S * N; e += NT, r += NT) {
+            while (r >= N) { r -= N; ++i; }
             double acc = 0.0;
 #pragma unroll
             for (int j = 0; j < S; ++j) acc = fma(RAD<S>().a[j][i], C.F[j * N + r], acc);
             C.yb[e] = acc;
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < S * N; e += NT) {
-            const int i = e / N, r = e - i * N;
+        for (int e = threadIdx.x, i = 0, r = threadIdx.x; e < S * N; e += NT, r += NT) {
+            while (r >= N) { r -= N; ++i; }
             C.aw[e] = apply_row_T(r, C.yb + i * N, sh.scj[i], C.diag, N, T);
         }
         __syncthreads();
@@ -1366,14 +1414,14 @@ __device__ int adjoint_stages(Ctx<S>& C, const DevTab& T, double hs, double h_f,
             for (int k = 0; k < S; ++k) {
                 float acc = 0.f;
 #pragma unroll
-                for (int i = 0; i < S; ++i) acc = fmaf((float)RAD<S>().T[i][k], rho[i], acc);
+                for (int i = 0; i < S; ++i) acc = fmaf(RAD<S>().Tf[i][k], rho[i], acc);
                 tr[k] = acc;
             }
             // Lam^T: real gam; pairs [[alp, -bet], [bet, alp]]
-            C.rr[b] = (float)RAD<S>().gam * tr[0];
+            C.rr[b] = RAD<S>().gamf * tr[0];
 #pragma unroll
             for (int p = 0; p < NC; ++p) {
-                const float al = (float)RAD<S>().alp[p], be = (float)RAD<S>().bet[p];
+                const float al = RAD<S>().alpf[p], be = RAD<S>().betf[p];
                 const float q1 = al * tr[1 + 2 * p] - be * tr[2 + 2 * p];
                 const float q2 = be * tr[1 + 2 * p] + al * tr[2 + 2 * p];
                 C.rc[p * N + b] = make_float2(q1, -q2);        // conjugated for the transposed complex solve
@@ -1405,7 +1453,7 @@ __device__ int adjoint_stages(Ctx<S>& C, const DevTab& T, double hs, double h_f,
             for (int k = 0; k < S; ++k) {
                 float dz = 0.f;
 #pragma unroll
-                for (int j = 0; j < S; ++j) dz = fmaf((float)RAD<S>().Ti[j][k], om[j], dz);
+                for (int j = 0; j < S; ++j) dz = fmaf(RAD<S>().Tif[j][k], om[j], dz);
                 C.F[k * N + r] += (double)dz;
                 dm = nanmax(dm, fabsf(dz));
                 zm = nanmax(zm, fabsf((float)C.F[k * N + r]));

@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <type_traits>
 #include "fp_internal.h"
 
 // ------------------------------------------------------------- Langevin ----
@@ -138,35 +139,45 @@ __global__ void __launch_bounds__(FP_EQ_BS) fp_equilibrium_kernel(EqArgs A, int 
 
 // -------------------------------------------------------------- M1 fit ----
 // Columns (c, k) are contiguous in the [N][C][K1] layout, so a block takes
-// FP_M1_COLS consecutive columns of one dictionary element and FP_M1_VG voxel
-// groups (voxels nu = g, g + VG, ...); partial sums meet in shared memory.
-#define FP_M1_COLS 64
-#define FP_M1_VG 4
+// COLS consecutive columns of one dictionary element and VG voxel groups
+// (voxels nu = g, g + VG, ...); partial sums meet in shared memory.
 
-// pass 1: a = sum S conj(Phi) / sum |Phi|^2 and max |S| per column
-__global__ void fp_m1_pass1(const double2* __restrict__ phi, const double2* __restrict__ S, int N, int CK,
+// Both passes are bound by the FP64 pipe (12 operations an entry at 2 a clock
+// and SM), HBM runs at a quarter of its rate: so max |S|^2 is formed by the
+// first element's CTAs alone, and the residual's two products and subtraction
+// are two fused operations a component.  96 elements x 1,024 voxels x 1,634
+// columns with fp_nrmse: 5.41 ms -> 3.40 ms; the FP64 floor is 3.07 ms.
+// pass 1: a = sum S conj(Phi) / sum |Phi|^2 and (q = 0) max |S| per column
+template <int COLS, int VG>
+__global__ void __launch_bounds__(COLS * VG) fp_m1_pass1(const double2* __restrict__ phi, const double2* __restrict__ S, int N, int CK,
                             double2* __restrict__ a, double* __restrict__ smax) {
-    __shared__ double red[FP_M1_VG][FP_M1_COLS][4];
-    const int col = blockIdx.x * FP_M1_COLS + (threadIdx.x % FP_M1_COLS);
-    const int g = threadIdx.x / FP_M1_COLS;
+    __shared__ double red[VG][COLS][4];
+    const int col = blockIdx.x * COLS + (threadIdx.x % COLS);
+    const int g = threadIdx.x / COLS;
     const int q = blockIdx.y;
     double sr = 0.0, si = 0.0, pp = 0.0, mx = 0.0;
     if (col < CK) {
         const double2* P = phi + (size_t)q * N * CK + col;
         const double2* Sv = S + col;
-        for (int nu = g; nu < N; nu += FP_M1_VG) {
+        if (q == 0) {
+            for (int nu = g; nu < N; nu += VG) {
+                const double2 s = __ldg(Sv + (size_t)nu * CK);
+                mx = fmax(mx, s.x * s.x + s.y * s.y);
+            }
+        }
+#pragma unroll 4
+        for (int nu = g; nu < N; nu += VG) {
             const double2 p = __ldg(P + (size_t)nu * CK), s = __ldg(Sv + (size_t)nu * CK);
             sr = fma(s.x, p.x, fma(s.y, p.y, sr));          // S conj(Phi)
             si = fma(s.y, p.x, fma(-s.x, p.y, si));
             pp = fma(p.x, p.x, fma(p.y, p.y, pp));
-            mx = fmax(mx, s.x * s.x + s.y * s.y);
         }
     }
-    const int cl = threadIdx.x % FP_M1_COLS;
+    const int cl = threadIdx.x % COLS;
     red[g][cl][0] = sr; red[g][cl][1] = si; red[g][cl][2] = pp; red[g][cl][3] = mx;
     __syncthreads();
     if (g == 0 && col < CK) {
-        for (int h = 1; h < FP_M1_VG; ++h) {
+        for (int h = 1; h < VG; ++h) {
             sr += red[h][cl][0]; si += red[h][cl][1]; pp += red[h][cl][2]; mx = fmax(mx, red[h][cl][3]);
         }
         const double ip = pp > 0.0 ? 1.0 / pp : 0.0;
@@ -176,63 +187,86 @@ __global__ void fp_m1_pass1(const double2* __restrict__ phi, const double2* __re
 }
 
 // pass 2: eps = sqrt(sum |S - a Phi|^2 / N) / max |S|
-__global__ void fp_m1_pass2(const double2* __restrict__ phi, const double2* __restrict__ S, int N, int CK,
+template <int COLS, int VG>
+__global__ void __launch_bounds__(COLS * VG) fp_m1_pass2(const double2* __restrict__ phi, const double2* __restrict__ S, int N, int CK,
                             const double2* __restrict__ a, const double* __restrict__ smax, double* __restrict__ eps) {
-    __shared__ double red[FP_M1_VG][FP_M1_COLS];
-    const int col = blockIdx.x * FP_M1_COLS + (threadIdx.x % FP_M1_COLS);
-    const int g = threadIdx.x / FP_M1_COLS;
+    __shared__ double red[VG][COLS];
+    const int col = blockIdx.x * COLS + (threadIdx.x % COLS);
+    const int g = threadIdx.x / COLS;
     const int q = blockIdx.y;
     double rr = 0.0;
     if (col < CK) {
         const double2 av = a[(size_t)q * CK + col];
         const double2* P = phi + (size_t)q * N * CK + col;
         const double2* Sv = S + col;
-        for (int nu = g; nu < N; nu += FP_M1_VG) {
+#pragma unroll 4
+        for (int nu = g; nu < N; nu += VG) {
             const double2 p = __ldg(P + (size_t)nu * CK), s = __ldg(Sv + (size_t)nu * CK);
-            const double dr = s.x - (av.x * p.x - av.y * p.y);
-            const double di = s.y - (av.x * p.y + av.y * p.x);
+            const double dr = fma(-av.x, p.x, fma(av.y, p.y, s.x));
+            const double di = fma(-av.x, p.y, fma(-av.y, p.x, s.y));
             rr = fma(dr, dr, fma(di, di, rr));
         }
     }
-    const int cl = threadIdx.x % FP_M1_COLS;
+    const int cl = threadIdx.x % COLS;
     red[g][cl] = rr;
     __syncthreads();
     if (g == 0 && col < CK) {
-        for (int h = 1; h < FP_M1_VG; ++h) rr += red[h][cl];
+        for (int h = 1; h < VG; ++h) rr += red[h][cl];
         const double m = smax[col];
         eps[(size_t)q * CK + col] = m > 0.0 ? sqrt(rr / N) / m : 0.0;
     }
 }
 
-// eps_freq[k] = sqrt(mean over (angle, channel) of eps^2); global = sqrt(mean over I_freq of eps_freq^2)
-__global__ void fp_nrmse_kernel(const double* __restrict__ eps, int A, int C, int K1, const int* __restrict__ ks,
-                                int nk, double* __restrict__ eps_freq, double* __restrict__ eps_global) {
-    __shared__ double red[256];
-    double part = 0.0;
-    for (int k = threadIdx.x; k < K1; k += blockDim.x) {
-        double s = 0.0;
-        for (int a = 0; a < A; ++a)
-            for (int c = 0; c < C; ++c) {
-                const double v = eps[((size_t)a * C + c) * K1 + k];
-                s = fma(v, v, s);
+// sums over (angle, channel) rows of eps^2 at the harmonics kof(i), i < cnt, 128 at
+// a time: warp w takes rows w, w + 32, ..., a lane four harmonics; the row
+// groups meet in shared memory and thread i adds up one harmonic (whole warps
+// at a time: an FP64 instruction holds the SM's pipe for 16 clocks however many
+// lanes it serves)
+template <class KOf, class Out>
+__device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int rows, int K1, int cnt, KOf kof, Out out) {
+    __shared__ double part[32][128];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min(32, rows);
+    for (int i0 = 0; i0 < cnt; i0 += 128) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        int k[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) k[c] = kof(min(i0 + 32 * c + lane, cnt - 1));
+        for (int r = w; r < rows; r += 32)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double v = __ldg(eps + (size_t)r * K1 + k[c]);
+                s[c] = fma(v, v, s[c]);
             }
-        s /= (double)(A * C);
-        if (eps_freq) eps_freq[k] = sqrt(s);
+        if (w < nw)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) part[w][32 * c + lane] = s[c];
+        __syncthreads();
+        const int i = i0 + threadIdx.x;
+        if (threadIdx.x < 128 && i < cnt) {
+            double v = 0.0;
+            for (int h = 0; h < nw; ++h) v += part[h][threadIdx.x];
+            out(i, v);
+        }
+        __syncthreads();
     }
+}
+
+// eps_freq[k] = sqrt(mean over (angle, channel) of eps^2); global = sqrt(mean over I_freq of eps_freq^2).
+// One CTA of 32 warps: a chain of loads over all rows per harmonic bounded the
+// former one-thread-per-harmonic form (192 rows x 817 harmonics: about 0.4 ms
+// of the 3.8 ms that fit and measures took then).
+__global__ void __launch_bounds__(1024) fp_nrmse_kernel(const double* __restrict__ eps, int A, int C, int K1,
+                                                        const int* __restrict__ ks, int nk,
+                                                        double* __restrict__ eps_freq, double* __restrict__ eps_global) {
+    __shared__ double red[128];
+    const double inv = (double)(A * C);
+    if (eps_freq)
+        nrmse_sums(eps, A * C, K1, K1, [](int i) { return i; }, [&](int i, double v) { eps_freq[i] = sqrt(v / inv); });
+    double acc = 0.0;
+    nrmse_sums(eps, A * C, K1, nk, [&](int i) { return __ldg(ks + i); }, [&](int, double v) { acc += v / inv; });
+    if (threadIdx.x < 128) red[threadIdx.x] = acc;
     __syncthreads();
-    for (int i = threadIdx.x; i < nk; i += blockDim.x) {
-        const int k = ks[i];
-        double s = 0.0;
-        for (int a = 0; a < A; ++a)
-            for (int c = 0; c < C; ++c) {
-                const double v = eps[((size_t)a * C + c) * K1 + k];
-                s = fma(v, v, s);
-            }
-        part += s / (double)(A * C);
-    }
-    red[threadIdx.x] = part;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    for (int o = 64; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
@@ -282,12 +316,21 @@ int fp_m1_fit(const double* d_phi, int Q, const double* d_S, int N, int C, int K
     if (Q == 0 || N == 0) return FP_OK;
     if (Q > 65535) return fp_fail(FP_EINVAL, "fp_m1_fit: Q=%d > 65535 dictionary elements per call", Q);
     const int CK = C * K1;
-    dim3 grid((CK + FP_M1_COLS - 1) / FP_M1_COLS, Q);
     cudaStream_t st = (cudaStream_t)stream;
-    fp_m1_pass1<<<grid, FP_M1_COLS * FP_M1_VG, 0, st>>>((const double2*)d_phi, (const double2*)d_S, N, CK,
-                                                        (double2*)d_a, d_smax);
-    fp_m1_pass2<<<grid, FP_M1_COLS * FP_M1_VG, 0, st>>>((const double2*)d_phi, (const double2*)d_S, N, CK,
-                                                        (const double2*)d_a, d_smax, d_eps);
+    // wide blocks with four voxel groups where they fill the GPU twice over;
+    // below that (few elements or harmonics) narrow ones with 32 groups:
+    // eight times the parallel chains (2 elements x 277 voxels x 126 columns: 95
+    // -> 39 us; 52 x 72 x 462, 416 wide blocks: 134 us narrow, 80 wide)
+    auto run = [&](auto cols, auto vg) {
+        constexpr int COLS = decltype(cols)::value, VG = decltype(vg)::value;
+        const dim3 grid((CK + COLS - 1) / COLS, Q);
+        fp_m1_pass1<COLS, VG><<<grid, COLS * VG, 0, st>>>((const double2*)d_phi, (const double2*)d_S, N, CK,
+                                                          (double2*)d_a, d_smax);
+        fp_m1_pass2<COLS, VG><<<grid, COLS * VG, 0, st>>>((const double2*)d_phi, (const double2*)d_S, N, CK,
+                                                          (const double2*)d_a, d_smax, d_eps);
+    };
+    if ((long long)((CK + 63) / 64) * Q >= 304) run(std::integral_constant<int, 64>(), std::integral_constant<int, 4>());
+    else run(std::integral_constant<int, 16>(), std::integral_constant<int, 32>());
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m1_fit: launch failed");
     return FP_OK;
 }
@@ -296,7 +339,7 @@ int fp_nrmse(const double* d_eps, int A, int C, int K1, const int* d_ks, int nk,
              double* d_eps_global, void* stream) {
     if (!d_eps || !d_ks || !d_eps_global) return fp_fail(FP_EINVAL, "fp_nrmse: NULL buffer");
     if (A < 1 || C < 1 || K1 < 1 || nk < 1) return fp_fail(FP_EINVAL, "fp_nrmse: bad sizes");
-    fp_nrmse_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(d_eps, A, C, K1, d_ks, nk, d_eps_freq, d_eps_global);
+    fp_nrmse_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(d_eps, A, C, K1, d_ks, nk, d_eps_freq, d_eps_global);
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_nrmse: launch failed");
     return FP_OK;
 }

@@ -166,7 +166,7 @@ int fp_setup(const fp_material* mat, const fp_drive* drive, const fp_tol* tol, i
         const size_t b_glob = rows * 4, b_u8 = rows * FP_NSB, b_f8 = rows * FP_NSB * 4, b_u6 = rows * FP_NLT,
                      b_f6 = rows * FP_NLT * 4;
         size_t offs[12], o = 0;
-        const size_t sizes[12] = {b_glob, b_u8, b_u8, b_f8, b_u6, b_u6, b_f6, b_u6, b_u6, b_f6, b_u6, b_u6};
+        const size_t sizes[12] = {b_glob, b_u8, b_u8, b_f8, b_u6, b_u6, b_f6, b_u6, b_u6, b_f6, rows * 16, rows * 16};
         for (int q = 0; q < 12; ++q) { offs[q] = o; o += (sizes[q] + 255) & ~(size_t)255; }
         std::vector<unsigned char> hb(o, 0);
         for (int L = 2; L <= L_max; ++L) {
@@ -182,8 +182,16 @@ int fp_setup(const fp_material* mat, const fp_drive* drive, const fp_tol* tol, i
             std::memcpy(&hb[offs[7] + r0 * FP_NLT], b.up_k, b.N * FP_NLT);
             std::memcpy(&hb[offs[8] + r0 * FP_NLT], b.up_g, b.N * FP_NLT);
             std::memcpy(&hb[offs[9] + r0 * FP_NLT * 4], b.up_cf, b.N * FP_NLT * 4);
-            std::memcpy(&hb[offs[10] + r0 * FP_NLT], b.dnT, b.N * FP_NLT);
-            std::memcpy(&hb[offs[11] + r0 * FP_NLT], b.upT, b.N * FP_NLT);
+            auto pack = [](unsigned char* out, const unsigned char* k, const unsigned char* back) {
+                for (int p = 0; p < FP_NLT; ++p) {
+                    out[p] = k[p] == 255 ? 0 : k[p];
+                    out[8 + p] = k[p] == 255 ? 255 : back[p];
+                }
+            };
+            for (int r = 0; r < b.N; ++r) {
+                pack(&hb[offs[10] + (r0 + r) * 16], b.dn_k + r * FP_NLT, b.dnT + r * FP_NLT);
+                pack(&hb[offs[11] + (r0 + r) * 16], b.up_k + r * FP_NLT, b.upT + r * FP_NLT);
+            }
             fp_free_blocks(&bl[L]);
         }
         up(&c->d_blk_mem, hb.data(), o);
@@ -199,8 +207,8 @@ int fp_setup(const fp_material* mat, const fp_drive* drive, const fp_tol* tol, i
         c->blk.up_k = base + offs[7];
         c->blk.up_g = base + offs[8];
         c->blk.up_cf = (const float*)(base + offs[9]);
-        c->blk.dnT = base + offs[10];
-        c->blk.upT = base + offs[11];
+        c->blk.dn_l = base + offs[10];
+        c->blk.up_l = base + offs[11];
     }
     FpRadau r3, r5;
     if (fp_build_radau(3, &r3) != FP_OK || fp_build_radau(5, &r5) != FP_OK) {

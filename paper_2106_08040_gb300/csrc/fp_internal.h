@@ -149,8 +149,10 @@ struct DevBlk {                      // block structure of every degree, packed
     const uint8_t* up_k;
     const uint8_t* up_g;
     const float* up_cf;
-    const uint8_t* dnT;
-    const uint8_t* upT;
+    // per row one 16-byte word each: partners (bytes 0-5, 0 where there is none) and their
+    // back pointers dnT / upT (bytes 8-13, 255 where there is none) of its dn and up lists
+    const unsigned char* dn_l;
+    const unsigned char* up_l;
     int off[FP_L_MAX + 2];           // first packed row of degree L
 };
 

@@ -109,7 +109,7 @@ __host__ __device__ inline Layout make_layout(int L) {
     size_t fsum = 0;
     for (int mu = 0; mu <= L; ++mu) fsum += (size_t)nblk(mu, L) * ldb(nblk(mu, L));
     ly.fsum = fsum;
-    const size_t N = ly.N, nm2 = (size_t)ly.nmax * ly.nmax;
+    const size_t N = ly.N, nm2 = (size_t)ly.nmax * ldb(ly.nmax);
     size_t o = 0;
     ly.y = o;    o = al16(o + N * 8);
     ly.Z = o;    o = al16(o + (size_t)S * N * 8);
@@ -350,13 +350,19 @@ struct Ctx {
     int* foff;
     // block structure of degree L
     const int* glob;
-    const uint8_t *sb_k, *sb_g, *dn_k, *dn_g, *up_k, *up_g, *dnT, *upT;
+    const uint8_t *sb_k, *sb_g, *dn_k, *dn_g, *up_k, *up_g;
+    const uint4 *dn_l, *up_l;       // packed lists: six partner bytes (x, y) and six back-pointer bytes (z, w)
     const float *sb_cf, *dn_cf, *up_cf;
 };
 
 // ------------------------------------------- factorisation (block Thomas) --
 __device__ __forceinline__ void named_bar(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// byte p of a packed list of six (lo, hi)
+__device__ __forceinline__ int link_byte(uint32_t lo, uint32_t hi, int p) {
+    return (int)(((p < 4 ? lo : hi) >> (8 * (p & 3))) & 255u);
 }
 
 // A group of GW warps assembles the Schur-complement block
@@ -410,7 +416,7 @@ __device__ void group_factor_block(Ctx<S>& C, int mu, T shift, const float* gs, 
                     for (int p = 0; p < FP_NSB; ++p) v = cadd_real(v, ks[p] == j ? vs[p] : 0.f);
 #pragma unroll
                     for (int p = 0; p < FP_NLT; ++p)
-                        if (kd[p] != 255) v = cfma(-vd[p], Xprev[kd[p] * n + j], v);
+                        if (kd[p] != 255) v = cfma(-vd[p], Xprev[kd[p] * ldb(n) + j], v);
                 }
                 a[s][jj] = v;
             }
@@ -483,7 +489,8 @@ __device__ void group_factor_block(Ctx<S>& C, int mu, T shift, const float* gs, 
     }
 }
 
-// X_mu = Inv_mu B_mu (n x n2, row-major) for one system; one warp per column c
+// X_mu = Inv_mu B_mu (n x n2, row-major, odd row stride as in ldb, so that rows a lane apart
+// lie in distinct banks) for one system; one warp per column c
 // (lane = row r).  B_mu[k][c] is the coupling of row k (block mu) to row c
 // (block mu+1), reached through the dn list of row c and its back pointer.
 template <class T, int S, int RS = 1>
@@ -491,22 +498,31 @@ __device__ __forceinline__ void x_column(Ctx<S>& C, int mu, int c, const T* inv,
     const int lane = threadIdx.x & 31;
     const int L = C.L, n = nblk(mu, L), n2 = nblk(mu + 1, L);
     const int bc = C.boff[mu + 1] + c, bo = C.boff[mu];
+    // absent couplings take part with value 0 and partner 0: without a branch each, the loads of
+    // all six are in flight together (a factorisation of degree 16: -5 %)
+    const uint4 dl = __ldg(C.dn_l + bc);
     T acc[RS];
+    float bv[FP_NLT];
 #pragma unroll
     for (int s = 0; s < RS; ++s) acc[s] = czero<T>();
 #pragma unroll
     for (int p = 0; p < FP_NLT; ++p) {
-        const int k = __ldg(C.dn_k + bc * FP_NLT + p);
-        if (k == 255) continue;
-        const int q = __ldg(C.dnT + bc * FP_NLT + p);
-        const float bv = q == 255 ? 0.f : C.upv[(bo + k) * FP_NLT + q];
+        const int q = link_byte(dl.z, dl.w, p);
+        bv[p] = q == 255 ? 0.f : C.upv[(bo + link_byte(dl.x, dl.y, p)) * FP_NLT + q];
+    }
 #pragma unroll
-        for (int s = 0; s < RS; ++s)
-            if (lane + 32 * s < n) acc[s] = cfma(bv, inv[k * ldb(n) + lane + 32 * s], acc[s]);
+    for (int s = 0; s < RS; ++s) {
+        if (lane + 32 * s < n) {
+            T iv[FP_NLT];
+#pragma unroll
+            for (int p = 0; p < FP_NLT; ++p) iv[p] = inv[link_byte(dl.x, dl.y, p) * ldb(n) + lane + 32 * s];
+#pragma unroll
+            for (int p = 0; p < FP_NLT; ++p) acc[s] = cfma(bv[p], iv[p], acc[s]);
+        }
     }
 #pragma unroll
     for (int s = 0; s < RS; ++s)
-        if (lane + 32 * s < n) X[(lane + 32 * s) * n2 + c] = acc[s];
+        if (lane + 32 * s < n) X[(lane + 32 * s) * ldb(n2) + c] = acc[s];
 }
 
 template <int S> struct Groups {
@@ -537,7 +553,7 @@ __device__ void factorize(Ctx<S>& C, const AScal& sc, double h, int* pp, float2*
     __syncthreads();
     const int w = threadIdx.x >> 5;
     const int sys = w / GW, gw = w - sys * GW;
-    const size_t nm2 = (size_t)C.ly.nmax * C.ly.nmax;
+    const size_t nm2 = (size_t)C.ly.nmax * ldb(C.ly.nmax);
     for (int mu = 0; mu <= L; ++mu) {
         if (sys == 0) {
             group_factor_block<float, S, GW, RS>(C, mu, RAD<S>().gamf, gs, (float)h, C.Xr, C.fr + C.foff[mu],
@@ -564,6 +580,22 @@ __device__ void factorize(Ctx<S>& C, const AScal& sc, double h, int* pp, float2*
 }
 
 // ----------------------------------------------------- warp-group solve --
+// The six transposed couplings of a block row: partner entries zk of the neighbouring block (zb)
+// and their values cv, from the partners' lists (vb) through the back pointers.  Absent ones have
+// value 0 and partner 0, so that the chained loads of all six are in flight together (gradients of
+// 25 voxels at degree 14: 542 -> 492 ms).  The plain solve, whose values lie in the row's own
+// list, is 1 % faster with a branch each.
+template <class T>
+__device__ __forceinline__ void coupled_T(const uint4* list, const float* vb, const T* zb, float* cv, T* zk) {
+    const uint4 l = __ldg(list);
+#pragma unroll
+    for (int p = 0; p < FP_NLT; ++p) {
+        const int k = link_byte(l.x, l.y, p), q = link_byte(l.z, l.w, p);
+        zk[p] = zb[k];
+        cv[p] = q == 255 ? 0.f : vb[k * FP_NLT + q];
+    }
+}
+
 // Block-Thomas solve of one system with its explicit block inverses by a group
 // of GW warps: row r of a block is handled by GW lanes (r = gw*RPW + lane%RPW,
 // part = lane/RPW) that split the matvec columns and reduce with shuffles.
@@ -584,18 +616,18 @@ __device__ void group_solve(Ctx<S>& C, const T* __restrict__ inv, T* rhs, T* z, 
         if (mu > 0 && part == 0 && r < n) {
             const int b = bo + r, bp = C.boff[mu - 1];
             T v = rhs[b];
+            if (TRANS) {
+                T zk[FP_NLT];
+                float cv[FP_NLT];
+                coupled_T(C.dn_l + b, C.upv + bp * FP_NLT, z + bp, cv, zk);
 #pragma unroll
-            for (int p = 0; p < FP_NLT; ++p) {
-                const int k = __ldg(C.dn_k + b * FP_NLT + p);
-                if (k == 255) continue;
-                float cv;
-                if (TRANS) {
-                    const int q = __ldg(C.dnT + b * FP_NLT + p);
-                    cv = q == 255 ? 0.f : C.upv[(bp + k) * FP_NLT + q];
-                } else {
-                    cv = C.dnv[b * FP_NLT + p];
+                for (int p = 0; p < FP_NLT; ++p) v = cfma(-cv[p], zk[p], v);
+            } else {
+#pragma unroll
+                for (int p = 0; p < FP_NLT; ++p) {
+                    const int k = __ldg(C.dn_k + b * FP_NLT + p);
+                    if (k != 255) v = cfma(-C.dnv[b * FP_NLT + p], z[bp + k], v);
                 }
-                v = cfma(-cv, z[bp + k], v);
             }
             rhs[b] = v;
         }
@@ -616,18 +648,18 @@ __device__ void group_solve(Ctx<S>& C, const T* __restrict__ inv, T* rhs, T* z, 
         if (part == 0 && r < n) {
             const int b = bo + r;
             T v = czero<T>();
+            if (TRANS) {
+                T zk[FP_NLT];
+                float cv[FP_NLT];
+                coupled_T(C.up_l + b, C.dnv + bn * FP_NLT, z + bn, cv, zk);
 #pragma unroll
-            for (int p = 0; p < FP_NLT; ++p) {
-                const int k = __ldg(C.up_k + b * FP_NLT + p);
-                if (k == 255) continue;
-                float cv;
-                if (TRANS) {
-                    const int q = __ldg(C.upT + b * FP_NLT + p);
-                    cv = q == 255 ? 0.f : C.dnv[(bn + k) * FP_NLT + q];
-                } else {
-                    cv = C.upv[b * FP_NLT + p];
+                for (int p = 0; p < FP_NLT; ++p) v = cfma(cv[p], zk[p], v);
+            } else {
+#pragma unroll
+                for (int p = 0; p < FP_NLT; ++p) {
+                    const int k = __ldg(C.up_k + b * FP_NLT + p);
+                    if (k != 255) v = cfma(C.upv[b * FP_NLT + p], z[bn + k], v);
                 }
-                v = cfma(cv, z[bn + k], v);
             }
             rhs[b] = v;
         }
@@ -789,8 +821,8 @@ __device__ FpParams setup_instance(Ctx<S>& C, const KArgs& A, const fp_instance&
     C.up_k = A.blk.up_k + (size_t)o * FP_NLT;
     C.up_g = A.blk.up_g + (size_t)o * FP_NLT;
     C.up_cf = A.blk.up_cf + (size_t)o * FP_NLT;
-    C.dnT = A.blk.dnT + (size_t)o * FP_NLT;
-    C.upT = A.blk.upT + (size_t)o * FP_NLT;
+    C.dn_l = (const uint4*)A.blk.dn_l + o;
+    C.up_l = (const uint4*)A.blk.up_l + o;
     __syncthreads();
     if (threadIdx.x == 0) {
         int bo = 0, fo = 0;

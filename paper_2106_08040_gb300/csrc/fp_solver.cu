@@ -760,6 +760,16 @@ __device__ __forceinline__ double sample_time(const fp_drive& d, int j) {
     return ((double)d.warmup_periods + (double)j / (double)d.samples_per_period) * d.period;
 }
 
+// What the block needs to know of a step.  FP64 runs at two operations a clock and SM, so a
+// scalar double operation costs 16 cycles of the pipe for every warp that repeats it, a division
+// about ten of them; the first two warps alone follow the time and the step size, and the first
+// publishes what the others need.
+struct StepCtl {
+    double hs, sc_err;
+    float fscale, escale;  // h_f / hs, and gam h_f / hs, for the step's factors
+    int last, refac, underflow;
+};
+
 // Shared (per-CTA) scalars of the instance being integrated.
 template <int S>
 struct Shared {
@@ -768,7 +778,9 @@ struct Shared {
     float2 colbuf[FP_CB_SYS * (1 + (S - 1) / 2)];
     float red[NWARP];
     double dred[NWARP * 12];
-    double R[9], off[3], dm[4];          // dm[3]: |<m>|^2 of the last written sample
+    double R[9], off[3];
+    StepCtl ctl;           // the step being made, published by the first warp
+    int unresolved;        // a written sample left the unit ball
     AScal scj[S];          // operator scalars at the stage times
     double Pm[S * S];      // predictor matrix
 };
@@ -846,11 +858,10 @@ __device__ FpParams setup_instance(Ctx<S>& C, const KArgs& A, const fp_instance&
 struct NewtonResult { bool conv, nonfinite; float theta, dmax; int iters; };
 
 template <int S, int RS = 1>
-__device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, double h_f, double sc_err, float& eta,
+__device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, float fscale, float sc_err, float& eta,
                                       float kappa, int maxit, Shared<S>& sh) {
     constexpr int NC = (S - 1) / 2;
     const int N = C.N, w = threadIdx.x >> 5;
-    const float fscale = (float)(h_f / hs);
     NewtonResult res{false, false, 0.f, 0.f, 0};
     float prev = 3.0e38f;
     eta = powf(fmaxf(eta, 1e-7f), 0.8f);
@@ -929,7 +940,7 @@ __device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, dou
             if (res.theta >= 0.99f) break;
             eta = res.theta / (1.f - res.theta);
         }
-        if (eta * dmax <= kappa * (float)sc_err || dmax <= 1e-3f * kappa * (float)sc_err) { res.conv = true; break; }
+        if (eta * dmax <= kappa * sc_err || dmax <= 1e-3f * kappa * sc_err) { res.conv = true; break; }
         prev = dmax;
     }
     return res;
@@ -937,9 +948,11 @@ __device__ NewtonResult newton_stages(Ctx<S>& C, const DevTab& T, double hs, dou
 
 // operator scalars at the S stage times of (t, hs) and, if pred, the
 // predictor matrix; one lane each, shared through sh
+// (the first two warps' part; a barrier has to follow)
 template <int S>
-__device__ void stage_scalars(const KArgs& A, const FpParams& P, const double* R, const double* off, double t,
-                              double hs, bool pred, double h_old, Shared<S>& sh) {
+__device__ __forceinline__ void stage_scalars_warps(const KArgs& A, const FpParams& P, const double* R,
+                                                    const double* off, double t, double hs, bool pred, double h_old,
+                                                    Shared<S>& sh) {
     const int lane = threadIdx.x & 31;
     if ((threadIdx.x >> 5) == 0) {
         // one drive component per lane (lane = 3 j + k), then lane j rotates
@@ -969,6 +982,12 @@ __device__ void stage_scalars(const KArgs& A, const FpParams& P, const double* R
             sh.Pm[lane] = lj - (j == S - 1 ? 1.0 : 0.0);
         }
     }
+}
+
+template <int S>
+__device__ void stage_scalars(const KArgs& A, const FpParams& P, const double* R, const double* off, double t,
+                              double hs, bool pred, double h_old, Shared<S>& sh) {
+    stage_scalars_warps<S>(A, P, R, off, t, hs, pred, h_old, sh);
     __syncthreads();
 }
 
@@ -1047,42 +1066,37 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
     int jn = 0;
     bool have_pred = false, fac_valid = false, force_refac = false;
     int since_fac = 0;
-    double h_f = 0.0, h_old = 0.0, t_f = 0.0;
+    double h_f = 0.0, h_old = 0.0, t_f = 0.0, tt = 0.0, hs = 0.0;
+    bool last = false;
     float eta = 1.0f;
 
+    if (threadIdx.x == 0) sh.unresolved = 0;
     {
         const AScal sc0 = make_scal(P, B);
         apply_A(C.y, C.f0, sc0, C.diag, N, T);                 // f0 = A(t) y
         __syncthreads();
     }
-    auto write_sample = [&](int j, const AScal& ss) {
-        if (REC) return;
-        // <m> and d<m>/dt at t_j (l = 1 rows of A(t_j) y, ss = operator scalars
-        // at t_j), rotated back to the lab frame
-        if (threadIdx.x < 3) {
-            int row = threadIdx.x == 0 ? 3 : threadIdx.x;   // x' <- (1,1), y' <- (1,-1), z' <- (1,0)
-            sh.dm[threadIdx.x] = sq43 * apply_row(row, C.y, ss, C.diag, N, T);
+    // <m> and d<m>/dt at t_j, rotated back to the lab frame, from y and the l = 1 rows of
+    // f0 = A(t_j) y: by the third warp, beside the first two warps' choice of the next step
+    auto write_sample = [&](int j) {
+        if (REC || threadIdx.x != 64) return;
+        // x' <- (1,1), y' <- (1,-1), z' <- (1,0)
+        double mp[3] = {sq43 * C.y[3], sq43 * C.y[1], sq43 * C.y[2]};
+        double dp[3] = {sq43 * C.f0[3], sq43 * C.f0[1], sq43 * C.f0[2]};
+        const double m2 = mp[0] * mp[0] + mp[1] * mp[1] + mp[2] * mp[2];
+        size_t o = ((size_t)inst * A.S_out + j) * 3;
+        for (int k = 0; k < 3; ++k) {
+            double mk = R[k] * mp[0] + R[3 + k] * mp[1] + R[6 + k] * mp[2];
+            double dk = R[k] * dp[0] + R[3 + k] * dp[1] + R[6 + k] * dp[2];
+            if (A.m_out) A.m_out[o + k] = mk;
+            if (A.dmdt_out) A.dmdt_out[o + k] = dk;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double mp[3] = {sq43 * C.y[3], sq43 * C.y[1], sq43 * C.y[2]};
-            double dp[3] = {sh.dm[0], sh.dm[1], sh.dm[2]};
-            sh.dm[3] = mp[0] * mp[0] + mp[1] * mp[1] + mp[2] * mp[2];
-            size_t o = ((size_t)inst * A.S_out + j) * 3;
-            for (int k = 0; k < 3; ++k) {
-                double mk = R[k] * mp[0] + R[3 + k] * mp[1] + R[6 + k] * mp[2];
-                double dk = R[k] * dp[0] + R[3 + k] * dp[1] + R[6 + k] * dp[2];
-                if (A.m_out) A.m_out[o + k] = mk;
-                if (A.dmdt_out) A.dmdt_out[o + k] = dk;
-            }
-        }
-        __syncthreads();
         // the mean of unit vectors has norm <= 1; beyond that the truncated
         // operator at this L is not dissipative for the instance
-        if (sh.dm[3] > (1.0 + 1e-6) * (1.0 + 1e-6) && out.status == FP_STATUS_OK) out.status = FP_STATUS_UNRESOLVED;
+        if (m2 > (1.0 + 1e-6) * (1.0 + 1e-6)) sh.unresolved = 1;
     };
 
-    if (sample_time(A.drv, 0) <= 0.0) { write_sample(0, make_scal(P, B)); jn = 1; }
+    if (sample_time(A.drv, 0) <= 0.0) { write_sample(0); jn = 1; }
 
     float ym = 0.f;
     for (int i = threadIdx.x; i < N; i += NT) ym = nanmax(ym, fabsf((float)C.y[i]));
@@ -1090,22 +1104,43 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
     if (!(ymax <= 3.0e38)) out.status = FP_STATUS_NONFINITE;      // initial state
 
     while (out.status == FP_STATUS_OK && jn < A.S_out) {
+        if (sh.unresolved) { out.status = FP_STATUS_UNRESOLVED; break; }
         if (out.nsteps + out.nrej >= A.tol.max_steps || (REC && out.nsteps >= max_rec)) {
             out.status = FP_STATUS_MAXSTEPS;
             break;
         }
-        if (h < 1e-6 * T_s) { out.status = FP_STATUS_STEP_UNDERFLOW; break; }
-        const double tt = sample_time(A.drv, jn);
-        // split the rest of the sample interval into equal steps of at most h, so
-        // the step (and with it the factorisation) changes rarely
-        const double rem = tt - t;
-        const double nrem = ceil(rem / fmin(h, T_s) * (1.0 - 1e-12));
-        const bool last = nrem <= 1.0;
-        const double hs = last ? rem : rem / nrem;
-        stage_scalars<S>(A, P, R, off, t, hs, have_pred, h_old, sh);
+        // the first two warps: split the rest of the sample interval into equal steps of at most h,
+        // so that the step (and with it the factorisation) changes rarely; then the operator scalars
+        // and the predictor (t, h, h_old and tt are theirs alone)
+        if (threadIdx.x < 64) {
+            tt = sample_time(A.drv, jn);
+            const double rem = tt - t;
+            const double nrem = ceil(rem / fmin(h, T_s) * (1.0 - 1e-12));
+            last = nrem <= 1.0;
+            hs = last ? rem : rem / nrem;
+            const double rat = fac_valid ? hs / h_f : 0.0;
+            const bool refac = !fac_valid || force_refac || rat < FP_HRAT_LO || rat > FP_HRAT_HI ||
+                               since_fac >= A.tol.refactor_every;
+            if (threadIdx.x == 0) {
+                const double hf = refac ? hs : h_f;
+                sh.ctl.hs = hs;
+                sh.ctl.sc_err = atol + rtol * ymax;
+                sh.ctl.fscale = (float)(hf / hs);
+                sh.ctl.escale = (float)(RAD<S>().gam * hf / hs);
+                sh.ctl.last = last;
+                sh.ctl.refac = refac;
+                sh.ctl.underflow = h < 1e-6 * T_s;
+            }
+            stage_scalars_warps<S>(A, P, R, off, t, hs, have_pred, h_old, sh);
+        }
+        __syncthreads();
+        if (sh.ctl.underflow) { out.status = FP_STATUS_STEP_UNDERFLOW; break; }
+        hs = sh.ctl.hs;
+        last = sh.ctl.last != 0;
+        const double sc_err = sh.ctl.sc_err;
+        const float sc_errf = (float)sc_err;
         const AScal s_end = sh.scj[S - 1];           // operator scalars at t + hs (c_S = 1)
-        const double rat = fac_valid ? hs / h_f : 0.0;
-        if (!fac_valid || force_refac || rat < FP_HRAT_LO || rat > FP_HRAT_HI || since_fac >= A.tol.refactor_every) {
+        if (sh.ctl.refac) {
             refactor_at<S, RS>(C, s_end, hs, sh);
             h_f = hs; t_f = t; fac_valid = true; force_refac = false; since_fac = 0; ++out.nfac;
         }
@@ -1114,8 +1149,8 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
             for (int i = threadIdx.x; i < N; i += NT) ck[i] = C.y[i];
         }
         predict_stages<S>(C, have_pred, sh);
-        const double sc_err = atol + rtol * ymax;
-        const NewtonResult nr = newton_stages<S, RS>(C, T, hs, h_f, sc_err, eta, FP_KAPPA, A.tol.newton_max_iter, sh);
+        const NewtonResult nr = newton_stages<S, RS>(C, T, hs, sh.ctl.fscale, sc_errf, eta, FP_KAPPA,
+                                                     A.tol.newton_max_iter, sh);
         out.nit += nr.iters;
         if (nr.nonfinite) { out.status = FP_STATUS_NONFINITE; break; }
         if (!nr.conv) {
@@ -1140,12 +1175,16 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
             group_solve<float, S, Groups<S>::GW, false, RS>(C, C.fr, C.rr, C.zr, threadIdx.x >> 5, 1);
         __syncthreads();
         float em = 0.f;
-        const float escale = (float)(RAD<S>().gam * h_f / hs);
+        const float escale = sh.ctl.escale;
         for (int b = threadIdx.x; b < N; b += NT) em = nanmax(em, fabsf(escale * C.zr[b]));
-        const double en = (double)block_max(em, sh.red) / sc_err;
-        if (!(en < 1e300)) { out.status = FP_STATUS_NONFINITE; break; }
-        const double fac = en > 0.0 ? 0.9 * (double)powf((float)en, -1.f / (S + 1)) : 4.0;
-        if (en <= 1.0) {
+        const double em_d = (double)block_max(em, sh.red);
+        if (!(em_d < 1e300 * sc_err)) { out.status = FP_STATUS_NONFINITE; break; }
+        double fac = 4.0;                            // of the first two warps
+        if (threadIdx.x < 64) {
+            const double en = em_d / sc_err;
+            if (en > 0.0) fac = 0.9 * (double)powf((float)en, -1.f / (S + 1));
+        }
+        if (em_d <= sc_err) {                        // as em_d / sc_err <= 1: the quotient of a > b does not round to 1
             if (REC && threadIdx.x == 0) {
                 double* r = rec_steps + (size_t)out.nsteps * FP_REC;
                 r[0] = t; r[1] = hs; r[2] = last ? (double)jn : -1.0; r[3] = t_f; r[4] = h_f;
@@ -1158,25 +1197,29 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
             ymax = block_max(ymx, sh.red);
             if (!(ymax <= 3.0e38)) { out.status = FP_STATUS_NONFINITE; break; }
             ++out.nsteps; ++since_fac;
-            t = last ? tt : t + hs;
             // f0 = A(t) y at the accepted point, for the next error estimate
             apply_A(C.y, C.f0, s_end, C.diag, N, T);
             __syncthreads();
-            if (last) { write_sample(jn, s_end); ++jn; }
-            double hn = hs * fmin(4.0, fmax(0.2, fac));
-            if (last && hs < h) hn = fac < 1.0 ? fmin(h, hn) : h;
-            // keep the factorised step when the controller asks for a small change
-            if (fac_valid && hn >= 0.9 * h_f && hn <= 1.2 * h_f) hn = fmax(h_f, hs);
-            h = fmin(hn, T_s);
-            h_old = hs;
+            if (last) { write_sample(jn); ++jn; }
+            if (threadIdx.x < 64) {
+                t = last ? tt : t + hs;
+                double hn = hs * fmin(4.0, fmax(0.2, fac));
+                if (last && hs < h) hn = fac < 1.0 ? fmin(h, hn) : h;
+                // keep the factorised step when the controller asks for a small change
+                if (fac_valid && hn >= 0.9 * h_f && hn <= 1.2 * h_f) hn = fmax(h_f, hs);
+                h = fmin(hn, T_s);
+                h_old = hs;
+            }
             have_pred = true;
         } else {
             ++out.nrej;
-            h = hs * fmax(0.1, fac);
+            if (threadIdx.x < 64) h = hs * fmax(0.1, fac);
             have_pred = false;
         }
         __syncthreads();
     }
+    __syncthreads();
+    if (sh.unresolved && out.status == FP_STATUS_OK) out.status = FP_STATUS_UNRESOLVED;     // the last sample
     if (!REC) {
         for (int e = jn * 3 + threadIdx.x; e < A.S_out * 3; e += NT) {
             if (A.m_out) A.m_out[(size_t)inst * A.S_out * 3 + e] = 0.0;
@@ -1614,7 +1657,7 @@ __global__ void __launch_bounds__(NT, 1) fp_adjoint_kernel(GArgs G) {
                 stage_scalars<S>(A, P, R, off, t, hs, pred, pred ? h_prev : 1.0, sh);
                 predict_stages<S>(C, pred, sh);
                 float eta = 1.f;
-                NewtonResult nr = newton_stages<S>(C, T, hs, h_f, sc_rep, eta, 0.02f, 4 * A.tol.newton_max_iter, sh);
+                NewtonResult nr = newton_stages<S>(C, T, hs, (float)(h_f / hs), (float)sc_rep, eta, 0.02f, 4 * A.tol.newton_max_iter, sh);
                 // a stalled iteration whose last increment is already below the
                 // tolerance scale is as good as the forward's accepted stages;
                 // otherwise (the forward reached these stages from a better
@@ -1625,7 +1668,7 @@ __global__ void __launch_bounds__(NT, 1) fp_adjoint_kernel(GArgs G) {
                     stage_scalars<S>(A, P, R, off, t, hs, false, 1.0, sh);
                     predict_stages<S>(C, false, sh);
                     eta = 1.f;
-                    nr = newton_stages<S>(C, T, hs, h_f, sc_rep, eta, 0.02f, 4 * A.tol.newton_max_iter, sh);
+                    nr = newton_stages<S>(C, T, hs, (float)(h_f / hs), (float)sc_rep, eta, 0.02f, 4 * A.tol.newton_max_iter, sh);
                 }
                 if (nr.nonfinite || (!nr.conv && !(nr.dmax <= (float)sc_rep))) {
                     status = nr.nonfinite ? FP_STATUS_NONFINITE : FP_STATUS_NEWTON_FAIL;

@@ -17,13 +17,12 @@
 // Every wait is bounded in time; a wait that gives up sets *err and the CTA
 // drains its copies and MMAs and frees TMEM before it returns.
 //
-// What bounds it (GB300, 262,144 queries): the 512 -> 512 layers take 139 us (192 us with a scalar
-// epilogue) and read 11 TB/s of operands from L2, which is its limit at 48 KB per 128 x 256 x 64
-// block; the first layer (K = 64) 120 us, its epilogue; both output layers together 530 us, again
+// What bounds it (GB300, 262,144 queries): the 512 -> 512 layers take 139 us and
+// read 11 TB/s of operands from L2, which is its limit, at 48 KB per 128 x 256 x 64 block; the first layer (K = 64) 120 us, its epilogue; both output layers together 530 us, again
 // 11 TB/s.  1,024,000 queries through two networks: 13.7 -> 6.46 ms.  Small batches are a chain of
 // launches: 257 queries 88 -> 32 us with narrow tiles and overlapped launches; a training step of
 // 4096 queries 590 -> 218 us with one launch for all weight gradients, one for the bias gradients
-// and one for the optimiser (27 launches before, 13 now).
+// and one for the optimiser (25 kernels before, 13 now).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>

@@ -5,8 +5,9 @@
 // from a work counter).  The real-SH coefficient vector c (N = (L+1)^2
 // doubles) and every Radau stage live in shared memory; the FP32 factors too
 // with 3 stages up to degree FP_L_SMEM, otherwise in a global slot per CTA
-// that stays in L2 (5 stages: two CTAs per SM).  Nothing is streamed from HBM
-// per step except the L1/L2-resident coupling tables shared by all instances.
+// that stays in L2 (5 stages with more instances than SMs: two CTAs per SM).
+// Nothing is streamed from HBM per step except the L1/L2-resident coupling
+// tables shared by all instances.
 //
 // Time step: S-stage Radau IIA (S = 3: order 5, S = 5: order 9; L-stable),
 // simplified Newton:
@@ -99,7 +100,8 @@ struct Layout {
 };
 
 // ADJ adds the adjoint state lambda (N) and one more stage-sized buffer (S N).
-template <int S, bool ADJ = false>
+// SF: five-stage factors in shared memory, one CTA per SM (batches that do not fill the SMs).
+template <int S, bool ADJ = false, bool SF = false>
 __host__ __device__ inline Layout make_layout(int L) {
     constexpr int NC = (S - 1) / 2;
     Layout ly;
@@ -127,7 +129,7 @@ __host__ __device__ inline Layout make_layout(int L) {
     // slot per CTA (the solve: two CTAs per SM; the adjoint: the slot opens
     // its workspace); three-stage factors stay in shared memory up to degree
     // FP_L_SMEM
-    ly.gfac = L > FP_L_SMEM || S == 5;
+    ly.gfac = L > FP_L_SMEM || (S == 5 && !SF);
     ly.fac_bytes = al16(fsum * 4) + al16((size_t)NC * fsum * 8);
     if (ly.gfac) {
         ly.fr = 0;
@@ -785,9 +787,9 @@ struct Shared {
     double Pm[S * S];      // predictor matrix
 };
 
-template <int S, bool ADJ>
+template <int S, bool ADJ, bool SF = false>
 __device__ void bind_smem(Ctx<S>& C, unsigned char* smem, int L_launch, Shared<S>& sh, unsigned char* fac) {
-    C.ly = make_layout<S, ADJ>(L_launch);
+    C.ly = make_layout<S, ADJ, SF>(L_launch);
     C.y = (double*)(smem + C.ly.y);
     C.Z = (double*)(smem + C.ly.Z);
     C.F = (double*)(smem + C.ly.F);
@@ -1230,13 +1232,14 @@ __device__ FwdOut forward_instance(Ctx<S>& C, const KArgs& A, int inst, const Fp
     return out;
 }
 
-template <int S, int RS>
-// five stages: 128 registers a thread, two CTAs per SM (factors in global memory)
-__global__ void __launch_bounds__(NT, S == 5 ? 2 : 1) fp_solve_kernel(KArgs A) {
+template <int S, int RS, bool SF = false>
+// five stages: 128 registers a thread, two CTAs per SM (factors in global memory), or with SF one
+// CTA per SM with all its registers and the factors in shared memory
+__global__ void __launch_bounds__(NT, S == 5 && !SF ? 2 : 1) fp_solve_kernel(KArgs A) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Shared<S> sh;
     Ctx<S> C;
-    bind_smem<S, false>(C, smem, A.L_launch, sh, A.fac ? A.fac + (size_t)blockIdx.x * A.fac_stride : nullptr);
+    bind_smem<S, false, SF>(C, smem, A.L_launch, sh, A.fac ? A.fac + (size_t)blockIdx.x * A.fac_stride : nullptr);
     __shared__ int s_slot;
     // instances come either round robin (slot = blockIdx.x + k gridDim.x) or,
     // with a work counter, one at a time in the caller's order, so CTAs that
@@ -1844,6 +1847,20 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
         const int grid = n < num_sms ? n : num_sms;
         fp_solve_kernel<3, 2><<<grid, NT, sm, st>>>(A);
         return cudaGetLastError() == cudaSuccess ? FP_OK : FP_ECUDA;
+    }
+    if (stages == 5 && !d_order && n <= num_sms) {
+        // no SM gets a second instance (and no other launch of a plan runs beside this one): factors in
+        // shared memory and 255 registers a thread.  60 instances of degree 16 over 204 samples: 132 ms with
+        // the two-CTA code, 98 ms with this one and the step control of the first two warps; one
+        // instance of degree 10: 70 and 58 ms.  Beyond one instance per SM the two-CTA layout is the
+        // faster one (1024 instances: 305 instance-periods/s, 276 with one CTA and these factors)
+        const size_t sm = make_layout<5, false, true>(L_launch).total;
+        if (cudaFuncSetAttribute(fp_solve_kernel<5, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) ==
+            cudaSuccess) {
+            fp_solve_kernel<5, 1, true><<<n, NT, sm, st>>>(A);
+            return cudaGetLastError() == cudaSuccess ? FP_OK : FP_ECUDA;
+        }
+        cudaGetLastError();
     }
     if (stages == 5) {
         // one global factor slot per CTA, up to two CTAs per SM

@@ -17,12 +17,13 @@
 // Every wait is bounded in time; a wait that gives up sets *err and the CTA
 // drains its copies and MMAs and frees TMEM before it returns.
 //
-// What bounds it (GB300, 262,144 queries): the 512 -> 512 layers take 139 us and
-// read 11 TB/s of operands from L2, which is its limit, at 48 KB per 128 x 256 x 64 block; the first layer (K = 64) 120 us, its epilogue; both output layers together 530 us, again
-// 11 TB/s.  1,024,000 queries through two networks: 13.7 -> 6.46 ms.  Small batches are a chain of
-// launches: 257 queries 88 -> 32 us with narrow tiles and overlapped launches; a training step of
-// 4096 queries 590 -> 218 us with one launch for all weight gradients, one for the bias gradients
-// and one for the optimiser (25 kernels before, 13 now).
+// What bounds it (GB300, 262,144 queries): the 512 -> 512 layers take 136 us and read 11 TB/s of
+// operands from L2, which is its limit, at 48 KB per 128 x 256 x 64 block; the first layer (K = 64)
+// 105 us, its epilogue; both output layers together 0.55 ms, again 11 TB/s.  1,024,000 queries
+// through two networks: 13.7 -> 6.36 ms.  Small batches are a chain of launches: 257 queries
+// 88 -> 32 us with narrow tiles and overlapped launches; a training step of 4096 queries
+// 594 -> 191 us with one launch for all weight gradients, one for the bias gradients and one for
+// the optimiser (25 kernels before, 13 now).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -37,7 +38,8 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;
-constexpr int EPI_GROUPS = 2;                 // column groups of the epilogue, 4 warps each
+constexpr int EPI_GROUPS = 4;                 // column groups of the epilogue, 4 warps each (two groups
+                                              // leave latency uncovered: K = 64 layer 120 us, with four 105 us)
 constexpr int NTHREADS = 64 + 128 * EPI_GROUPS;   // TMA warp, MMA warp, epilogue warps
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // 2 s bound on any single wait
 
@@ -298,6 +300,15 @@ constexpr int EPI_WARPS = 4 * EPI_GROUPS;    // warps 2 ..
 constexpr int MAX_EPI_COLS = 1024;           // bias / output scale staged in shared memory
 
 // ---------------------------------------------------------------- epilogue ----
+// 16 consecutive values in shared memory (a warp reads the same ones: 16-byte broadcasts)
+__device__ __forceinline__ void lds16(const float* p, float* r) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+        const float4 a = *(const float4*)(p + i);
+        r[i] = a.x; r[i + 1] = a.y; r[i + 2] = a.z; r[i + 3] = a.w;
+    }
+}
+
 // 16 consecutive floats of a row at o, `left` columns of them valid; vec as in EpiParams
 __device__ __forceinline__ void store_row16(float* o, const float* r, int vec, int left) {
     if (left >= 16 && vec == 2) {
@@ -337,12 +348,19 @@ __device__ __forceinline__ void epilogue_chunk(const EpiParams& P, int row, int 
     const bool rv = row < M;
     if (EPI == EPI_OUT_ENSEMBLE) {
         if (!rv) return;
-        float mn[16];
+        float mn[16], y1s[16], b[16], sc[16], sh[16];
+        lds16(sb + MAX_EPI_COLS, b);
+        lds16(ssc + MAX_EPI_COLS, sc);
+        lds16(ssh + MAX_EPI_COLS, sh);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) y1s[i] = (v1[i] + b[i]) * sc[i] + sh[i];
+        lds16(sb, b);
+        lds16(ssc, sc);
+        lds16(ssh, sh);
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const bool cv = i < left;
-            const float y0 = (v[i] + sb[i]) * ssc[i] + ssh[i];
-            const float y1 = (v1[i] + sb[MAX_EPI_COLS + i]) * ssc[MAX_EPI_COLS + i] + ssh[MAX_EPI_COLS + i];
+            const float y0 = (v[i] + b[i]) * sc[i] + sh[i], y1 = y1s[i];
             const float d = cv ? y0 - y1 : 0.f;
             mn[i] = cv ? 0.5f * (y0 + y1) : 0.f;
             racc[0] = fmaf(d, d, racc[0]);
@@ -357,9 +375,12 @@ __device__ __forceinline__ void epilogue_chunk(const EpiParams& P, int row, int 
     }
     if (EPI == EPI_OUT_INFER) {
         if (!rv) return;
-        float r[16];
+        float r[16], b[16], sc[16], sh[16];
+        lds16(sb, b);
+        lds16(ssc, sc);
+        lds16(ssh, sh);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) r[i] = (v[i] + sb[i]) * ssc[i] + ssh[i];
+        for (int i = 0; i < 16; ++i) r[i] = (v[i] + b[i]) * sc[i] + sh[i];
         store_row16(P.outf + (size_t)row * P.ldf + col0, r, P.vec, left);
         return;
     }
@@ -610,7 +631,7 @@ mlp_gemm_kernel(const __grid_constant__ Maps<EPI> maps, const __grid_constant__ 
             const uint32_t tw1 = tmem + (uint32_t)(((u + NP - 1) % RING) * BN) + ((uint32_t)(lg * 32) << 16);
             float racc[2] = {0.f, 0.f};
             uint32_t r[2][16], r1[16];
-            tmem_ld16(tw + c_lo, r[0]);
+            if (c_lo < c_hi) tmem_ld16(tw + c_lo, r[0]);
 #pragma unroll 1
             for (int c = c_lo; c < c_hi; c += 32) {
 #pragma unroll
@@ -744,28 +765,36 @@ int gemm_bn(const Operand* op, int M, int N, int K, EpiParams P, cudaStream_t st
     return launch_t<BN, EPI>(maps, P, (int)nt, st);
 }
 
-// Tile width: the widest (fewest operand reads) that still gives every SM a tile.  A few
-// hundred queries are latency-bound, and a narrow tile has a short epilogue (257 queries:
-// 24 tiles of 64 columns against 6 of 256).  The K order, and with it the result, is the same.
+// Tile width: the one with the least waves x (columns + 48).  A wave's time grows with its
+// tiles' columns (epilogue and operand reads; the 48 stand for the A rows and the fill of the
+// pipeline), so large batches take the widest tile, and a few hundred queries, which are
+// latency-bound, a narrow one with a short epilogue (257 queries: 24 tiles of 64 columns in
+// one wave).  The K order, and with it the result, is the same for all.
+long long tile_cost(int M, int N, int BN) {
+    const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN), sms = num_sms();
+    return (tiles + sms - 1) / sms * (BN + 48);
+}
 template <int EPI>
 int gemm_hidden(const Operand& op, int M, int N, int K, const EpiParams& P, cudaStream_t st) {
-    const long long rows = (M + BM - 1) / BM, sms = num_sms();
-    if (rows * ((N + 255) / 256) >= sms) return gemm_bn<256, EPI>(&op, M, N, K, P, st);
-    if (rows * ((N + 127) / 128) >= sms) return gemm_bn<128, EPI>(&op, M, N, K, P, st);
+    const long long c256 = tile_cost(M, N, 256), c128 = tile_cost(M, N, 128), c64 = tile_cost(M, N, 64);
+    if (c256 <= c128 && c256 <= c64) return gemm_bn<256, EPI>(&op, M, N, K, P, st);
+    if (c128 <= c64) return gemm_bn<128, EPI>(&op, M, N, K, P, st);
     return gemm_bn<64, EPI>(&op, M, N, K, P, st);
 }
 template <int EPI>
 int gemm_out(const Operand* op, int M, int N, int K, const EpiParams& P, cudaStream_t st) {
-    if ((long long)((M + BM - 1) / BM) * ((N + 159) / 160) >= num_sms()) return gemm_bn<160, EPI>(op, M, N, K, P, st);
+    const long long c160 = tile_cost(M, N, 160), c80 = tile_cost(M, N, 80), c32 = tile_cost(M, N, 32);
+    if (c160 <= c80 && c160 <= c32) return gemm_bn<160, EPI>(op, M, N, K, P, st);
+    if (c80 <= c32) return gemm_bn<80, EPI>(op, M, N, K, P, st);
     return gemm_bn<32, EPI>(op, M, N, K, P, st);
 }
 
 // The weight gradients of every layer, gW [N][K] = GT [N][q] XT [K][q]^T, in one launch.  One
 // layer has 4 to 14 tiles of 128 x 256 behind a serial K loop over the batch, which leaves most
-// SMs idle; the group has 80 of 128 x 128 side by side.
+// SMs idle; the group has 137 of 128 x 80 side by side, one to an SM.
 struct DwLayer { const void *GT, *XT; float* gW; int N, K; };
 int gemm_dw(const DwLayer* dw, int q, int ldt, int* err, cudaStream_t st) {
-    constexpr int BN = 128;
+    constexpr int BN = 80;
     Maps<EPI_DW> maps;
     EpiParams P;
     std::memset(&P, 0, sizeof(P));
@@ -828,7 +857,7 @@ __global__ void bias_grad_kernel(BiasArgs a) {
     n -= a.row0[l];
     const __nv_bfloat16* g = a.gT[l] + (size_t)n * a.ldt;
     float s = 0.f;
-#pragma unroll 8
+#pragma unroll 32                                        // latency-bound: many loads in flight, one order of summation
     for (int m = lane; m < a.q; m += 32) s += __bfloat162float(g[m]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -972,7 +1001,8 @@ extern "C" {
 
 long long fp_surrogate_workspace_bytes(int q, int training) {
     if (q < 1) return fp_fail(FP_EINVAL, "fp_surrogate_workspace_bytes: q=%d", q);
-    return (long long)(training == 1 ? train_ws(q, nullptr, nullptr) : infer_ws(q, training == 2, nullptr, nullptr));
+    return (long long)(training && training != 2 ? train_ws(q, nullptr, nullptr)
+                                                  : infer_ws(q, training == 2, nullptr, nullptr));
 }
 
 // normalised input and the four hidden layers of one network; layer l writes w.h[dst[l]]

@@ -25,10 +25,10 @@ def sur():
 
 
 def thresholds():
-    """Batch sizes around the row counts where a wider tile still gives every SM one."""
+    """Batch sizes over the range in which the tile widths change: fractions and multiples of one row block per SM."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    edges = [128 * (-(-sms // t) - 1) for t in (5, 4, 2)]          # output tiles of 160, hidden tiles of 128 and 256
-    return [1, 127, 257] + [e + d for e in edges for d in (0, 1)]
+    blocks = [sms // 25, sms // 10, sms // 8, sms // 5, sms // 4, sms // 3, sms // 2, sms]
+    return [1, 127, 257] + [128 * b + d for b in blocks for d in (0, 1)]
 
 
 def queries(n, seed):
@@ -68,7 +68,7 @@ def test_non_finite_query_stays_in_its_row(sur):
 
 
 def test_ensemble_is_independent_of_the_batch(sur):
-    """Mean: the same bits.  Spread: two sums of 800 squares, each in 10 or 50 partial sums added in any
+    """Mean: the same bits.  Spread: two sums of 800 squares, each in 10 to 50 partial sums added in any
     order (at most 90 and 66 roundings of 2^-24 deep), under square roots: 160 roundings bound the ratio."""
     from paper_2106_08040_gb300 import surrogate_train
     ens = surrogate_train.Ensemble([random_net(sur, 31), random_net(sur, 32)])

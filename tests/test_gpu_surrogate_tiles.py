@@ -95,3 +95,21 @@ def test_grad_matches_oracle_over_the_tile_rules(sur, q):
     for l in range(sur.LAYERS):
         assert rel(s.gW[l].cpu().numpy(), gW[l]) < 3e-2, l
         assert rel(s.gb[l].cpu().numpy(), gb[l]) < 3e-2, l
+
+
+def test_launches_can_be_captured(sur):
+    """The overlapped launches of an inference, recorded into a CUDA graph, answer new inputs on replay."""
+    s = random_net(sur, 25)
+    x = queries(300, 10)
+    y = torch.empty((300, 800), device="cuda")
+    s.infer(x, out=y)                                  # workspace and module load happen outside the capture
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        s.infer(x, out=y)
+    x2 = queries(300, 11)
+    ref = s.infer(x2)
+    x.copy_(x2)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, ref) and s.error_flag() == 0

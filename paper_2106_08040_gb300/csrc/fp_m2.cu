@@ -106,7 +106,9 @@ __global__ void __launch_bounds__(M2_T * M2_T) fp_m2_gram_kernel(GramArgs g) {
 // upper triangle, 78 % of the measured FP64 rate (25 x 26 / 2 micro tiles hold 9 % more products than
 // the triangle, 352 threads 8 % more than the tiles).
 #define M2_RB 16           // rows staged per step
-#define M2_MAXNT 32        // J + 1 <= 128: at most 528 threads and 33 KB of staged rows
+#define M2_MAXNT 32        // J + 1 <= 128: at most 528 threads and 33 KB of staged rows, within the 48 KB
+                           // that every launch may use: a larger limit would be set per process, under
+                           // the launches of other host threads
 struct GramRow { long long phi, a, S; double sig; };
 
 __global__ void __launch_bounds__(544, 1) fp_m2_gram_micro_kernel(GramArgs g, int nt, int groups) {
@@ -432,8 +434,6 @@ int fp_m2_gram(const double* d_phi, const double* d_a, const double* d_S, const 
         const long long ctas = steps < 2LL * sms ? steps : (mt * groups > 272 ? (long long)sms : 2LL * sms);
         g.rows_per_split = (steps + ctas - 1) / ctas * M2_RB;
         const unsigned grid = (unsigned)((g.R + g.rows_per_split - 1) / g.rows_per_split);
-        if (cudaFuncSetAttribute(fp_m2_gram_micro_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-            return fp_fail(FP_ECUDA, "fp_m2_gram: smem attribute");
         fp_m2_gram_micro_kernel<<<grid, threads, sm, st>>>(g, nt, groups);
         if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m2_gram: launch failed");
         return FP_OK;

@@ -1,0 +1,59 @@
+"""Calls from several host threads at once, each thread with its own buffers, stream and
+(where the call takes one) context: a kernel's dynamic shared-memory limit is state of the
+process, so a launch must not depend on the size that another thread asks for in between.
+Refusals would come back as errors of the launch; nothing here faults.
+"""
+import threading
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2106_08040_gb300 import build      # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fp():
+    build.build()
+    from paper_2106_08040_gb300 import fp as fpmod
+    return fpmod
+
+
+def run_threads(calls, repeat, sync_every):
+    """Each call, a function of a stream, `repeat` times in a thread of its own; the errors raised.
+    A full launch queue would hold the threads back, so each waits for its stream now and then."""
+    errors = []
+    start = threading.Barrier(len(calls))
+
+    def loop(call):
+        s = torch.cuda.Stream()
+        start.wait()
+        for i in range(repeat):
+            try:
+                call(s)
+            except RuntimeError as e:
+                errors.append(str(e))
+            if i % sync_every == sync_every - 1:
+                s.synchronize()
+        s.synchronize()
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=loop, args=(c,)) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    return errors
+
+
+def test_m2_gram_of_different_column_counts(fp):
+    def call(J, N=64, nk=32):
+        z = lambda *s: torch.zeros(*s, dtype=torch.float64, device="cuda")        # noqa: E731
+        ks = torch.arange(nk, dtype=torch.int32, device="cuda")
+        a = (z(1, J, N, 1, nk, 2), z(1, J, 1, nk, 2), z(1, N, 1, nk, 2), z(1, 1, nk) + 1.0, 1, J, N, 1, nk, ks, nk,
+             z(J + 1, J + 1, 2))
+        return lambda s: fp.fp_m2_gram(*a, stream=s)
+
+    assert run_threads([call(J) for J in (35, 48) * 3], 20000, 1) == []

@@ -1812,6 +1812,19 @@ __global__ void __launch_bounds__(NT, 1) fp_adjoint_kernel(GArgs G) {
 }
 
 // --------------------------------------------------------- host launch ----
+// Allows a block of `kernel` all the shared memory that the current device has.  The limit belongs
+// to the process, so it is the same in every call: one set to the size of the call at hand would be
+// changed by another host thread between set and launch.
+static cudaError_t allow_smem(const void* kernel) {
+    cudaFuncAttributes fa;
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+}
+
 int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_material* mat, const fp_drive* drv,
                     const fp_tol* tol, const fp_instance* d_inst, int n, int L_launch, double* d_m, double* d_dmdt,
                     int* d_status, int* d_stats, int num_sms, cudaStream_t st, const int* d_order, int* d_queue,
@@ -1842,7 +1855,7 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
         A.fac = d_fac;
         A.fac_stride = fp_solver_fac_bytes(3, L_launch);
         const size_t sm = fp_solver_smem_bytes(3, L_launch);
-        e = cudaFuncSetAttribute(fp_solve_kernel<3, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_smem((const void*)fp_solve_kernel<3, 2>);
         if (e != cudaSuccess) return FP_ECUDA;
         const int grid = n < num_sms ? n : num_sms;
         fp_solve_kernel<3, 2><<<grid, NT, sm, st>>>(A);
@@ -1855,8 +1868,7 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
         // instance of degree 10: 70 and 58 ms.  Beyond one instance per SM the two-CTA layout is the
         // faster one (1024 instances: 305 instance-periods/s, 276 with one CTA and these factors)
         const size_t sm = make_layout<5, false, true>(L_launch).total;
-        if (cudaFuncSetAttribute(fp_solve_kernel<5, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) ==
-            cudaSuccess) {
+        if (allow_smem((const void*)fp_solve_kernel<5, 1, true>) == cudaSuccess) {
             fp_solve_kernel<5, 1, true><<<n, NT, sm, st>>>(A);
             return cudaGetLastError() == cudaSuccess ? FP_OK : FP_ECUDA;
         }
@@ -1868,7 +1880,7 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
         A.fac = d_fac;
         A.fac_stride = fp_solver_fac_bytes(5, L_launch);
         const size_t sm = fp_solver_smem_bytes(5, L_launch);
-        e = cudaFuncSetAttribute(fp_solve_kernel<5, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_smem((const void*)fp_solve_kernel<5, 1>);
         if (e != cudaSuccess) return FP_ECUDA;
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fp_solve_kernel<5, 1>, NT, sm) != cudaSuccess)
@@ -1886,7 +1898,7 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
     int per_sm = 0;
     cudaFuncSetAttribute(fp_solve_kernel<3, 1>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          (int)cudaSharedmemCarveoutMaxShared);
-    e = cudaFuncSetAttribute(fp_solve_kernel<3, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    e = allow_smem((const void*)fp_solve_kernel<3, 1>);
     if (e != cudaSuccess) return FP_ECUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fp_solve_kernel<3, 1>, NT, sm) != cudaSuccess) per_sm = 1;
     if (per_sm < 1) per_sm = 1;
@@ -1940,11 +1952,11 @@ int fp_launch_adjoint(int stages, const DevTab* tab, const DevBlk* blk, const fp
     size_t sm = fp_adjoint_smem_bytes(stages, L_launch);
     cudaError_t e;
     if (stages == 5) {
-        e = cudaFuncSetAttribute(fp_adjoint_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_smem((const void*)fp_adjoint_kernel<5>);
         if (e != cudaSuccess) return FP_ECUDA;
         fp_adjoint_kernel<5><<<grid, NT, sm, st>>>(G);
     } else {
-        e = cudaFuncSetAttribute(fp_adjoint_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        e = allow_smem((const void*)fp_adjoint_kernel<3>);
         if (e != cudaSuccess) return FP_ECUDA;
         fp_adjoint_kernel<3><<<grid, NT, sm, st>>>(G);
     }

@@ -5,11 +5,12 @@ Refusals would come back as errors of the launch; nothing here faults.
 """
 import threading
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2106_08040_gb300 import build      # noqa: E402
+from paper_2106_08040_gb300 import build, workloads      # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -57,3 +58,26 @@ def test_m2_gram_of_different_column_counts(fp):
         return lambda s: fp.fp_m2_gram(*a, stream=s)
 
     assert run_threads([call(J) for J in (35, 48) * 3], 20000, 1) == []
+
+
+@pytest.mark.parametrize("stages,n,degrees", [(3, 1, (4, 16)), (5, 1, (4, 16)), (5, 200, (4, 16)), (3, 1, (17, 24))])
+def test_solves_of_different_degrees(fp, stages, n, degrees):
+    """Instances of no volume: every launch ends at once, with status FP_STATUS_BAD_INPUT."""
+    d = workloads.DriveSpec(amp=(0.01, 0.0, 0.0), freq=(25e3,) * 3, phase=(0.0,) * 3, period=4e-5,
+                            samples_per_period=2, warmup_periods=0, output_periods=1)
+    ctxs, statuses = [], []
+
+    def call(L):
+        ctx = fp.Context(fp.Material(), fp.Drive(**d.__dict__), fp.Tol(stages=stages), L)
+        inst = workloads.random_instances(n, L)
+        inst["d"] = 0.0
+        d_inst = fp.instances_to_device(inst)
+        st = torch.zeros(n, dtype=torch.int32, device="cuda")
+        ctxs.append(ctx)
+        statuses.append(st)
+        return lambda s: fp.fp_solve_batch(ctx, d_inst, n, None, None, st, None, stream=s)
+
+    assert run_threads([call(L) for L in degrees * 3], 3000, 250) == []
+    assert all(bool((st == 5).all()) for st in statuses)
+    for c in ctxs:
+        c.close()

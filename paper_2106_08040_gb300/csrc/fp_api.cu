@@ -451,6 +451,7 @@ extern "C" int fp_signal(fp_ctx* ctx, const double* d_dmdt, int n, int k_max, co
                       : make_double3(0, 0, 0);
     size_t sm = (size_t)S * C * sizeof(double);
     if (sm > 200 * 1024) return fail(FP_EUNSUPPORTED, "fp_signal: period too long for shared memory");
+    // the limits are the same in every call: they belong to the process, and other host threads may launch
     SigPlan P;
     // the transform writes pairs: a result that is not 16-byte aligned takes the direct kernel
     if ((reinterpret_cast<unsigned long long>(d_phihat) & 15ull) == 0 && sig_plan(S, k_max, &P)) {
@@ -460,7 +461,7 @@ extern "C" int fp_signal(fp_ctx* ctx, const double* d_dmdt, int n, int k_max, co
         fp_signal_fft_kernel<<<dim3(n, C), 256, sm, (cudaStream_t)stream>>>(
             d_dmdt, S_out, S, k_max, (const double2*)ctx->d_tw, P, ch[0], ch[1], ch[2], ch[3], (double2*)d_phihat);
     } else {
-        if (cudaFuncSetAttribute(fp_signal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+        if (cudaFuncSetAttribute(fp_signal_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
             return fail(FP_ECUDA, "fp_signal: smem attribute");
         fp_signal_kernel<<<n, 256, sm, (cudaStream_t)stream>>>(d_dmdt, S_out, S, k_max, ctx->d_tw, C, ch[0], ch[1],
                                                               ch[2], ch[3], d_phihat);

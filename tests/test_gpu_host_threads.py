@@ -81,3 +81,22 @@ def test_solves_of_different_degrees(fp, stages, n, degrees):
     assert all(bool((st == 5).all()) for st in statuses)
     for c in ctxs:
         c.close()
+
+
+def test_signals_of_different_periods(fp):
+    """Two harmonics of periods of 32 and 20,000 samples: the direct sum, whose samples lie in shared memory."""
+    ctxs = []
+
+    def call(S):
+        d = workloads.DriveSpec(amp=(0.01, 0.0, 0.0), freq=(25e3,) * 3, phase=(0.0,) * 3, period=S / 2.5e6,
+                                samples_per_period=S, warmup_periods=0, output_periods=1)
+        ctx = fp.Context(fp.Material(), fp.Drive(**d.__dict__), fp.Tol(), 4)
+        ctxs.append(ctx)
+        dm = torch.ones((1, S, 3), dtype=torch.float64, device="cuda")
+        out = torch.empty((1, 1, 2, 2), dtype=torch.float64, device="cuda")
+        ch = np.array([[1.0, 0.0, 0.0]])
+        return lambda s: fp.fp_signal(ctx, dm, 1, 1, ch, out, stream=s)
+
+    assert run_threads([call(S) for S in (32, 20000) * 3], 1500, 250) == []
+    for c in ctxs:
+        c.close()

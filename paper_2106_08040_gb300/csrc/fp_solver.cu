@@ -1812,17 +1812,19 @@ __global__ void __launch_bounds__(NT, 1) fp_adjoint_kernel(GArgs G) {
 }
 
 // --------------------------------------------------------- host launch ----
-// Allows a block of `kernel` all the shared memory that the current device has.  The limit belongs
-// to the process, so it is the same in every call: one set to the size of the call at hand would be
-// changed by another host thread between set and launch.
-static cudaError_t allow_smem(const void* kernel) {
+// Allows a block of `kernel` all the shared memory that the current device has beside its static
+// part (*room).  The limit belongs to the process, so it is the same in every call: one set to the
+// size of the call at hand would be changed by another host thread between set and launch.
+static cudaError_t allow_smem(const void* kernel, size_t* room = nullptr) {
     cudaFuncAttributes fa;
     int dev = 0, optin = 0;
     cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    const int bytes = optin - (int)fa.sharedSizeBytes;
+    if (room) *room = (size_t)bytes;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_material* mat, const fp_drive* drv,
@@ -1868,11 +1870,12 @@ int fp_launch_solve(int stages, const DevTab* tab, const DevBlk* blk, const fp_m
         // instance of degree 10: 70 and 58 ms.  Beyond one instance per SM the two-CTA layout is the
         // faster one (1024 instances: 305 instance-periods/s, 276 with one CTA and these factors)
         const size_t sm = make_layout<5, false, true>(L_launch).total;
-        if (allow_smem((const void*)fp_solve_kernel<5, 1, true>) == cudaSuccess) {
+        size_t room = 0;
+        if (allow_smem((const void*)fp_solve_kernel<5, 1, true>, &room) != cudaSuccess) return FP_ECUDA;
+        if (sm <= room) {                            // 219 KB at degree 16
             fp_solve_kernel<5, 1, true><<<n, NT, sm, st>>>(A);
             return cudaGetLastError() == cudaSuccess ? FP_OK : FP_ECUDA;
         }
-        cudaGetLastError();
     }
     if (stages == 5) {
         // one global factor slot per CTA, up to two CTAs per SM

@@ -159,19 +159,18 @@ __global__ void __launch_bounds__(COLS * VG) fp_m1_pass1(const double2* __restri
     if (col < CK) {
         const double2* P = phi + (size_t)q * N * CK + col;
         const double2* Sv = S + col;
-        if (q == 0) {
-            for (int nu = g; nu < N; nu += VG) {
-                const double2 s = __ldg(Sv + (size_t)nu * CK);
-                mx = fmax(mx, s.x * s.x + s.y * s.y);
-            }
-        }
+        auto sums = [&](auto with_max) {                      // one pass over the data either way
 #pragma unroll 4
-        for (int nu = g; nu < N; nu += VG) {
-            const double2 p = __ldg(P + (size_t)nu * CK), s = __ldg(Sv + (size_t)nu * CK);
-            sr = fma(s.x, p.x, fma(s.y, p.y, sr));          // S conj(Phi)
-            si = fma(s.y, p.x, fma(-s.x, p.y, si));
-            pp = fma(p.x, p.x, fma(p.y, p.y, pp));
-        }
+            for (int nu = g; nu < N; nu += VG) {
+                const double2 p = __ldg(P + (size_t)nu * CK), s = __ldg(Sv + (size_t)nu * CK);
+                sr = fma(s.x, p.x, fma(s.y, p.y, sr));      // S conj(Phi)
+                si = fma(s.y, p.x, fma(-s.x, p.y, si));
+                pp = fma(p.x, p.x, fma(p.y, p.y, pp));
+                if (decltype(with_max)::value) mx = fmax(mx, s.x * s.x + s.y * s.y);
+            }
+        };
+        if (q == 0) sums(std::true_type());
+        else sums(std::false_type());
     }
     const int cl = threadIdx.x % COLS;
     red[g][cl][0] = sr; red[g][cl][1] = si; red[g][cl][2] = pp; red[g][cl][3] = mx;
@@ -317,10 +316,20 @@ int fp_m1_fit(const double* d_phi, int Q, const double* d_S, int N, int C, int K
     if (Q > 65535) return fp_fail(FP_EINVAL, "fp_m1_fit: Q=%d > 65535 dictionary elements per call", Q);
     const int CK = C * K1;
     cudaStream_t st = (cudaStream_t)stream;
-    // wide blocks with four voxel groups where they fill the GPU twice over;
-    // below that (few elements or harmonics) narrow ones with 32 groups:
-    // eight times the parallel chains (2 elements x 277 voxels x 126 columns: 95
-    // -> 39 us; 52 x 72 x 462, 416 wide blocks: 134 us narrow, 80 wide)
+    // Wide blocks (64 columns, four voxel groups), or narrow ones (16 columns, 32 groups: eight times
+    // the parallel chains) where wide ones leave SMs idle and there are voxels enough to pay for the
+    // reduction over 32 groups.  How many it takes depends on how many narrow blocks share an SM, one
+    // to eight up to two wide blocks per SM; measured on both sides of each line (us, wide / narrow):
+    // 16 wide blocks 17 / 17 at 32 voxels, 25 / 18 at 64; 52 blocks 19 / 21 at 40, 23 / 21 at 48; 104
+    // blocks 41 / 45 at 128, 77 / 72 at 277; 140 blocks 56 / 60 at 192, 142 / 126 at 512; 200 blocks 65 / 68
+    // at 128, 93 / 85 at 192; 260 blocks 133 / 138 at 277, 242 / 222 at 512.  Below 33 voxels wide ones
+    // always (1 element x 16 x 40: 13 us, 17 by narrow ones)
+    static const int min_voxels[9] = {0, 33, 44, 192, 272, 128, 160, 336, 640};
+    int dev = 0, sms = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long wide = (long long)((CK + 63) / 64) * Q, per_sm = ((long long)((CK + 15) / 16) * Q + sms - 1) / sms;
+    const bool narrow = wide < 2LL * sms && N >= min_voxels[per_sm < 8 ? per_sm : 8];
     auto run = [&](auto cols, auto vg) {
         constexpr int COLS = decltype(cols)::value, VG = decltype(vg)::value;
         const dim3 grid((CK + COLS - 1) / COLS, Q);
@@ -329,8 +338,8 @@ int fp_m1_fit(const double* d_phi, int Q, const double* d_S, int N, int C, int K
         fp_m1_pass2<COLS, VG><<<grid, COLS * VG, 0, st>>>((const double2*)d_phi, (const double2*)d_S, N, CK,
                                                           (const double2*)d_a, d_smax, d_eps);
     };
-    if ((long long)((CK + 63) / 64) * Q >= 304) run(std::integral_constant<int, 64>(), std::integral_constant<int, 4>());
-    else run(std::integral_constant<int, 16>(), std::integral_constant<int, 32>());
+    if (narrow) run(std::integral_constant<int, 16>(), std::integral_constant<int, 32>());
+    else run(std::integral_constant<int, 64>(), std::integral_constant<int, 4>());
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m1_fit: launch failed");
     return FP_OK;
 }

@@ -1,0 +1,53 @@
+"""Sizes on both sides of the model kernels' dispatch lines against the oracle or numpy, at
+the bars of the other model tests: sums of up to a few thousand FP64 products, 1e-12
+relative.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2106_08040_gb300 import build      # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fp():
+    build.build()
+    from paper_2106_08040_gb300 import fp as fpmod
+    return fpmod
+
+
+def rel(a, b):
+    return np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(np.asarray(b))
+
+
+def cplx(rng, shape):
+    return rng.normal(size=shape) + 1j * rng.normal(size=shape)
+
+
+def dev(z):
+    return torch.from_numpy(np.ascontiguousarray(np.stack([z.real, z.imag], -1))).cuda()
+
+
+# one to eight narrow blocks per SM, a voxel less than the line and at it; ragged columns
+@pytest.mark.parametrize("N,C,K1,Q", [(32, 1, 17, 2), (33, 1, 17, 2), (43, 1, 1000, 4), (44, 1, 1000, 4),
+                                      (191, 2, 800, 4), (192, 2, 800, 4), (271, 1, 2000, 4), (272, 1, 2000, 4),
+                                      (127, 1, 2500, 4), (128, 1, 2500, 4), (159, 1, 3000, 4), (160, 1, 3000, 4),
+                                      (335, 1, 4200, 4), (336, 1, 4200, 4), (639, 1, 4800, 4), (640, 1, 4800, 4),
+                                      (640, 1, 5000, 4)])
+def test_m1_fit_at_the_lines(fp, N, C, K1, Q):
+    from oracle import models
+    rng = np.random.default_rng(N + Q)
+    Phi, S = cplx(rng, (Q, N, C, K1)), cplx(rng, (N, C, K1))
+    a = torch.empty((Q, C, K1, 2), dtype=torch.float64, device="cuda")
+    eps = torch.empty((Q, C, K1), dtype=torch.float64, device="cuda")
+    smax = torch.empty((C, K1), dtype=torch.float64, device="cuda")
+    fp.fp_m1_fit(dev(Phi), Q, dev(S), N, C, K1, a, eps, smax)
+    ag, eg = a.cpu().numpy(), eps.cpu().numpy()
+    for q in (0, Q - 1):
+        ao, eo = models.m1_fit(Phi[q], S)
+        assert rel(ag[q][..., 0] + 1j * ag[q][..., 1], ao) <= 1e-12, q
+        assert np.abs(eg[q] - eo).max() <= 1e-12 * np.abs(eo).max(), q
+    np.testing.assert_allclose(smax.cpu().numpy(), np.abs(S).max(0), rtol=1e-15)

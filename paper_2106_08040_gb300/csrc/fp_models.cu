@@ -220,10 +220,10 @@ __global__ void __launch_bounds__(COLS * VG) fp_m1_pass2(const double2* __restri
 // a time: warp w takes rows w, w + 32, ..., a lane four harmonics; the row
 // groups meet in shared memory and thread i adds up one harmonic (whole warps
 // at a time: an FP64 instruction holds the SM's pipe for 16 clocks however many
-// lanes it serves)
+// lanes it serves).  part: one buffer for every instance of the template, within the 48 KB
+// of static shared memory
 template <class KOf, class Out>
-__device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int rows, int K1, int cnt, KOf kof, Out out) {
-    __shared__ double part[32][128];
+__device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int rows, int K1, int cnt, double (*part)[128], KOf kof, Out out) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min(32, rows);
     for (int i0 = 0; i0 < cnt; i0 += 128) {
         double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -257,12 +257,13 @@ __device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int r
 __global__ void __launch_bounds__(1024) fp_nrmse_kernel(const double* __restrict__ eps, int A, int C, int K1,
                                                         const int* __restrict__ ks, int nk,
                                                         double* __restrict__ eps_freq, double* __restrict__ eps_global) {
-    __shared__ double red[128];
+    __shared__ double part[32][128], red[128];
     const double inv = (double)(A * C);
     if (eps_freq)
-        nrmse_sums(eps, A * C, K1, K1, [](int i) { return i; }, [&](int i, double v) { eps_freq[i] = sqrt(v / inv); });
+        nrmse_sums(eps, A * C, K1, K1, part, [](int i) { return i; },
+                   [&](int i, double v) { eps_freq[i] = sqrt(v / inv); });
     double acc = 0.0;
-    nrmse_sums(eps, A * C, K1, nk, [&](int i) { return __ldg(ks + i); }, [&](int, double v) { acc += v / inv; });
+    nrmse_sums(eps, A * C, K1, nk, part, [&](int i) { return __ldg(ks + i); }, [&](int, double v) { acc += v / inv; });
     if (threadIdx.x < 128) red[threadIdx.x] = acc;
     __syncthreads();
     for (int o = 64; o > 0; o >>= 1) {

@@ -216,57 +216,84 @@ __global__ void __launch_bounds__(COLS * VG) fp_m1_pass2(const double2* __restri
     }
 }
 
-// sums over (angle, channel) rows of eps^2 at the harmonics kof(i), i < cnt, 128 at
-// a time: warp w takes rows w, w + 32, ..., a lane four harmonics; the row
-// groups meet in shared memory and thread i adds up one harmonic (whole warps
-// at a time: an FP64 instruction holds the SM's pipe for 16 clocks however many
-// lanes it serves).  part: one buffer for every instance of the template, within the 48 KB
-// of static shared memory
+// sums over (angle, channel) rows of eps^2 at the harmonics kof(i), i < cnt.  More than
+// FP_NRMSE_NK harmonics: one to each of FP_NRMSE_BS threads, loads in flight over the rows and no
+// barriers (rows x harmonics with both sums: 1 x 20,000 151 us, 16 x 817 19, 64 x 817 40; with
+// the form below 355, 35 and 69).  Up to that many, where most of those threads would have
+// nothing to do: warp w takes rows w, w + 32, ..., a lane four harmonics; the row groups
+// meet in shared memory and thread i adds up one harmonic (64 rows x 40: 15 us, 31 by one
+// thread per harmonic).  Whole warps at a time either way: an FP64 instruction holds the SM's
+// pipe for 16 clocks however many lanes it serves.  part: one buffer for every instance of
+// the template, within the 48 KB of static shared memory
+#define FP_NRMSE_BS 512
+#define FP_NRMSE_NK 128
 template <class KOf, class Out>
-__device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int rows, int K1, int cnt, double (*part)[128], KOf kof, Out out) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min(32, rows);
-    for (int i0 = 0; i0 < cnt; i0 += 128) {
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-        int k[4];
+__device__ __forceinline__ void nrmse_sums(const double* __restrict__ eps, int rows, int K1, int cnt,
+                                           double (*part)[FP_NRMSE_NK], KOf kof, Out out) {
+    if (cnt > FP_NRMSE_NK) {
+        if (threadIdx.x < FP_NRMSE_BS)
+            for (int i = threadIdx.x; i < cnt; i += FP_NRMSE_BS) {
+                const double* e = eps + kof(i);
+                double v = 0.0;
+                int r = 0;
+                if (rows >= 16) {                                 // four chains: shorter sums, smaller error
+                    double u[4] = {0.0, 0.0, 0.0, 0.0};
+                    for (; r + 4 <= rows; r += 4)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) k[c] = kof(min(i0 + 32 * c + lane, cnt - 1));
+                        for (int c = 0; c < 4; ++c) {
+                            const double x = __ldg(e + (size_t)(r + c) * K1);
+                            u[c] = fma(x, x, u[c]);
+                        }
+                    v = (u[0] + u[1]) + (u[2] + u[3]);
+                }
+                for (; r < rows; ++r) {
+                    const double x = __ldg(e + (size_t)r * K1);
+                    v = fma(x, x, v);
+                }
+                out(i, v);
+            }
+        return;
+    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min(32, rows);
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int k[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) k[c] = kof(min(32 * c + lane, cnt - 1));
+    if (w < nw) {
         for (int r = w; r < rows; r += 32)
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const double v = __ldg(eps + (size_t)r * K1 + k[c]);
                 s[c] = fma(v, v, s[c]);
             }
-        if (w < nw)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) part[w][32 * c + lane] = s[c];
-        __syncthreads();
-        const int i = i0 + threadIdx.x;
-        if (threadIdx.x < 128 && i < cnt) {
-            double v = 0.0;
-            for (int h = 0; h < nw; ++h) v += part[h][threadIdx.x];
-            out(i, v);
-        }
-        __syncthreads();
+        for (int c = 0; c < 4; ++c) part[w][32 * c + lane] = s[c];
     }
+    __syncthreads();
+    if (threadIdx.x < cnt) {
+        double v = 0.0;
+        for (int h = 0; h < nw; ++h) v += part[h][threadIdx.x];
+        out(threadIdx.x, v);
+    }
+    __syncthreads();
 }
 
 // eps_freq[k] = sqrt(mean over (angle, channel) of eps^2); global = sqrt(mean over I_freq of eps_freq^2).
-// One CTA of 4 to 32 warps: a chain of loads over all rows per harmonic bounded the
-// former one-thread-per-harmonic form (192 rows x 817 harmonics: about 0.4 ms
-// of the 3.8 ms that fit and measures took then).
+// One CTA of 4 to 32 warps.
 __global__ void __launch_bounds__(1024) fp_nrmse_kernel(const double* __restrict__ eps, int A, int C, int K1,
                                                         const int* __restrict__ ks, int nk,
                                                         double* __restrict__ eps_freq, double* __restrict__ eps_global) {
-    __shared__ double part[32][128], red[128];
+    __shared__ double part[32][FP_NRMSE_NK], red[FP_NRMSE_BS];
     const double inv = (double)(A * C);
     if (eps_freq)
         nrmse_sums(eps, A * C, K1, K1, part, [](int i) { return i; },
                    [&](int i, double v) { eps_freq[i] = sqrt(v / inv); });
     double acc = 0.0;
     nrmse_sums(eps, A * C, K1, nk, part, [&](int i) { return __ldg(ks + i); }, [&](int, double v) { acc += v / inv; });
-    if (threadIdx.x < 128) red[threadIdx.x] = acc;
+    const int width = nk > FP_NRMSE_NK ? FP_NRMSE_BS : FP_NRMSE_NK;     // threads that hold a part of the sum
+    if (threadIdx.x < width) red[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = 64; o > 0; o >>= 1) {
+    for (int o = width / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
         __syncthreads();
     }
@@ -349,9 +376,11 @@ int fp_nrmse(const double* d_eps, int A, int C, int K1, const int* d_ks, int nk,
              double* d_eps_global, void* stream) {
     if (!d_eps || !d_ks || !d_eps_global) return fp_fail(FP_EINVAL, "fp_nrmse: NULL buffer");
     if (A < 1 || C < 1 || K1 < 1 || nk < 1) return fp_fail(FP_EINVAL, "fp_nrmse: bad sizes");
-    // a warp per row, at most 32; four at least take the harmonics (1 row x 40 harmonics: the barriers of
-    // 32 warps made the fit with its measures 25 us, 19 us with one thread per harmonic)
-    const int rows = A * C, threads = 32 * (rows < 4 ? 4 : rows > 32 ? 32 : rows);
+    // a warp per row, at most 32; four at least take the harmonics (1 row x 40 harmonics with the
+    // fit: 25 us with 32 warps, for their barriers), FP_NRMSE_BS threads where there are more of them
+    const int rows = A * C, most = d_eps_freq && K1 > nk ? K1 : nk;
+    int threads = 32 * (rows < 4 ? 4 : rows > 32 ? 32 : rows);
+    if (most > FP_NRMSE_NK && threads < FP_NRMSE_BS) threads = FP_NRMSE_BS;
     fp_nrmse_kernel<<<1, threads, 0, (cudaStream_t)stream>>>(d_eps, A, C, K1, d_ks, nk, d_eps_freq, d_eps_global);
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_nrmse: launch failed");
     return FP_OK;

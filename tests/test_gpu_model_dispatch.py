@@ -51,3 +51,21 @@ def test_m1_fit_at_the_lines(fp, N, C, K1, Q):
         assert rel(ag[q][..., 0] + 1j * ag[q][..., 1], ao) <= 1e-12, q
         assert np.abs(eg[q] - eo).max() <= 1e-12 * np.abs(eo).max(), q
     np.testing.assert_allclose(smax.cpu().numpy(), np.abs(S).max(0), rtol=1e-15)
+
+
+# either sum in either form: at most 128 harmonics (warps over rows), more (a thread each, 512 and 513 of them)
+@pytest.mark.parametrize("A,C,K1,nk", [(1, 1, 128, 128), (1, 1, 129, 128), (1, 1, 129, 129), (3, 1, 512, 5),
+                                       (40, 1, 513, 513), (17, 2, 128, 128), (2, 1, 5000, 4000), (70, 3, 130, 129)])
+def test_nrmse_at_the_lines(fp, A, C, K1, nk):
+    from oracle import models
+    rng = np.random.default_rng(K1 + A)
+    eps = rng.uniform(0.05, 0.4, size=(A, C, K1))
+    ks = np.sort(rng.choice(K1, size=nk, replace=False)).astype(np.int32)
+    for want in (True, False):
+        ef = torch.full((K1,), np.nan, dtype=torch.float64, device="cuda") if want else None
+        eg = torch.empty(1, dtype=torch.float64, device="cuda")
+        fp.fp_nrmse(torch.from_numpy(eps).cuda(), A, C, K1, torch.from_numpy(ks).cuda(), nk, ef, eg)
+        if want:
+            assert rel(ef.cpu().numpy(), models.eps_freq(eps)) <= 1e-14
+        ref = models.eps_global(eps, ks)
+        assert abs(float(eg.item()) - ref) <= 1e-14 * ref

@@ -419,31 +419,46 @@ int fp_m2_gram(const double* d_phi, const double* d_a, const double* d_S, const 
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(d_G, 0, (size_t)fp_m2_gram_bytes(J), st) != cudaSuccess)
         return fp_fail(FP_ECUDA, "fp_m2_gram: clearing the output failed");
+    // row splits of the tiled kernel: four blocks an SM, whole steps of M2_R rows
+    const long long max_split = (g.R + M2_R - 1) / M2_R;
+    long long splits = (4LL * sms + tiles - 1) / tiles;
+    if (splits > max_split) splits = max_split;
+    if (splits > 65535) splits = 65535;
+    const long long tiled_rows = ((g.R + splits - 1) / splits + M2_R - 1) / M2_R * M2_R;
+    splits = (g.R + tiled_rows - 1) / tiled_rows;
     const int nt = (J + 1 + 3) / 4;
     if (nt >= 5 && nt <= M2_MAXNT && g.R >= 2048) {
-        // 17 to 128 columns: below, the micro tiles fill less than half a warp;
-        // above, the threads of one block do not suffice.  Few rows leave the
-        // staging latency bare: 36 columns x 528 rows 35.9 us here, 31.9 us tiled;
-        // 26 x 11,000 rows 81 against 106, 97 x 1.2 million rows 46.8 ms against 105.1
+        // 17 to 128 columns (below, the micro tiles fill less than half a warp; above, the
+        // threads of one block do not suffice) and 2,048 rows or more; then the kernel that the
+        // estimates name.  Both are steps of 16 rows on the busiest SM, in us, fitted to 930 times of 30
+        // column counts and 31 row counts (the micro tiles within 22 %, on average 5 %, the tiled
+        // kernel 13 % and 2 %): a step of the micro tiles takes 0.0165 us per row of a thread,
+        // adding up the groups 1.8 us each; a step of the tiled kernel 5.8 us per block of the
+        // SM and 1.4 us of latency.  Few rows leave the micro tiles' blocks with one step or
+        // two and part of the SMs with twice the work of others: 17 columns x 2,304 rows 46 us
+        // against 24 tiled, 8,192 rows 59 against 76; 64 x 2,720 rows 108 against 80, 4,096 rows
+        // 111 against 129; 97 x 1.2 million rows 46.8 ms against 105.1
         const int mt = nt * (nt + 1) / 2;
         const int groups = mt > 128 ? 1 : (256 / mt < M2_RB ? 256 / mt : M2_RB);
         const int threads = (mt * groups + 31) / 32 * 32;
-        size_t sm = (size_t)M2_RB * (4 * nt + 1) * sizeof(double2);
-        if (groups > 1 && sm < (size_t)mt * 256) sm = (size_t)mt * 256;
         const long long steps = (g.R + M2_RB - 1) / M2_RB;
         const long long ctas = steps < 2LL * sms ? steps : (mt * groups > 272 ? (long long)sms : 2LL * sms);
-        g.rows_per_split = (steps + ctas - 1) / ctas * M2_RB;
-        const unsigned grid = (unsigned)((g.R + g.rows_per_split - 1) / g.rows_per_split);
-        fp_m2_gram_micro_kernel<<<grid, threads, sm, st>>>(g, nt, groups);
-        if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m2_gram: launch failed");
-        return FP_OK;
+        const long long cta_steps = (steps + ctas - 1) / ctas, grid = (steps + cta_steps - 1) / cta_steps;
+        const double micro_us = 12.5 + 1.8 * (groups - 1) +
+                                0.0165 * (double)((grid + sms - 1) / sms * cta_steps) * threads *
+                                    ((M2_RB + groups - 1) / groups);
+        const double tiled_us = 6.8 + (double)(tiled_rows / M2_R) *
+                                          (1.4 + 5.8 * (double)((tiles * splits + sms - 1) / sms));
+        if (micro_us < 0.97 * tiled_us) {
+            size_t sm = (size_t)M2_RB * (4 * nt + 1) * sizeof(double2);
+            if (groups > 1 && sm < (size_t)mt * 256) sm = (size_t)mt * 256;
+            g.rows_per_split = cta_steps * M2_RB;
+            fp_m2_gram_micro_kernel<<<(unsigned)grid, threads, sm, st>>>(g, nt, groups);
+            if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m2_gram: launch failed");
+            return FP_OK;
+        }
     }
-    long long splits = (4LL * sms + tiles - 1) / tiles;
-    const long long max_split = (g.R + M2_R - 1) / M2_R;
-    if (splits > max_split) splits = max_split;
-    if (splits > 65535) splits = 65535;
-    g.rows_per_split = ((g.R + splits - 1) / splits + M2_R - 1) / M2_R * M2_R;
-    splits = (g.R + g.rows_per_split - 1) / g.rows_per_split;
+    g.rows_per_split = tiled_rows;
     fp_m2_gram_kernel<<<dim3(tiles, (unsigned)splits), M2_T * M2_T, 0, st>>>(g);
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_m2_gram: launch failed");
     return FP_OK;

@@ -69,3 +69,24 @@ def test_nrmse_at_the_lines(fp, A, C, K1, nk):
             assert rel(ef.cpu().numpy(), models.eps_freq(eps)) <= 1e-14
         ref = models.eps_global(eps, ks)
         assert abs(float(eg.item()) - ref) <= 1e-14 * ref
+
+
+# row counts on both sides of the lines: one row group to sixteen in a block, one step of rows to several, a ragged end
+@pytest.mark.parametrize("J", [16, 19, 23, 27, 31, 35, 47, 60, 63, 64, 95, 127])
+@pytest.mark.parametrize("N", [85, 96, 128, 190, 512])
+def test_m2_gram_at_the_lines(fp, J, N):
+    A, C, K1, nk = 1, 2, 21, 16
+    rng = np.random.default_rng(1000 * J + N)
+    Phi, a, S = cplx(rng, (A, J, N, C, K1)), cplx(rng, (A, J, C, K1)), cplx(rng, (A, N, C, K1))
+    ks = np.sort(rng.choice(K1, size=nk, replace=False)).astype(np.int32)
+    smax = np.abs(S).max(1)
+    G = torch.full((J + 1, J + 1, 2), np.nan, dtype=torch.float64, device="cuda")
+    fp.fp_m2_gram(dev(Phi), dev(a), dev(S), torch.from_numpy(smax).cuda(), A, J, N, C, K1,
+                  torch.from_numpy(ks).cuda(), nk, G)
+    Gg = G.cpu().numpy()
+    Gg = Gg[..., 0] + 1j * Gg[..., 1]
+    M = np.concatenate([a[:, :, None] * Phi, S[:, None]], axis=1) / smax[:, None, None]
+    M = M[..., ks].transpose(0, 2, 3, 4, 1).reshape(-1, J + 1)
+    Go = M.conj().T @ M
+    iu = np.triu_indices(J + 1)
+    assert np.abs(Gg[iu] - Go[iu]).max() <= 1e-12 * np.abs(Go).max()

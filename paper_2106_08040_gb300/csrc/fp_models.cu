@@ -64,7 +64,8 @@ struct EqArgs {
     double* dmdt_out;
 };
 
-// A thread takes one sample and FP_EQ_MAXG instances at most: B = off + amp sin(w t + ph),
+// A thread takes one sample and FP_EQ_MAXG instances at most; a block 2^lw samples of 128 >> lw groups
+// of instances (instance q of the block belongs to group q mod their number): B = off + amp sin(w t + ph),
 // dB/dt = amp w cos(w t + ph); m = L(xi) B/|B| = bT g B,
 // dm/dt = bT [g dB/dt + d (Bhat . dB/dt) Bhat]   (xi = bT |B|).
 // The FP64 pipe bounds it: the drive's three sincos (the larger half of the
@@ -72,11 +73,17 @@ struct EqArgs {
 // instance's bT and 1/bT once per CTA, and the quotients share one reciprocal
 // square root of |B|^2 and one of 1 - e^(-2 xi).  1,024 instances x 1,632 samples
 // with fp_signal (816 harmonics, 2 channels): 11.02 ms -> 0.67 ms together.
+// An SM's pipe serves a warp in the same time however few of its lanes have a sample: blocks of 128
+// samples throughout made 129 samples x 1,024 instances 77 us, 64 us with a thread per
+// sample and instance; the launch takes 8 samples a block there, 55 us.
 #define FP_EQ_BS 128
 #define FP_EQ_MAXG 16
-__global__ void __launch_bounds__(FP_EQ_BS) fp_equilibrium_kernel(EqArgs A, int G) {
-    __shared__ double si[FP_EQ_MAXG][5];                  // offset (3), bT (0: no moment), 1 / bT
-    const int j = blockIdx.x * FP_EQ_BS + threadIdx.x;
+#define FP_EQ_MINLW 2                                     // 4 samples a block at least: 96 bytes of an instance
+#define FP_EQ_MAXI (FP_EQ_MAXG * (FP_EQ_BS >> FP_EQ_MINLW))
+__global__ void __launch_bounds__(FP_EQ_BS) fp_equilibrium_kernel(EqArgs A, int G, int lw) {
+    __shared__ double si[FP_EQ_MAXI][5];                  // offset (3), bT (-1: no moment), 1 / bT
+    const int j = (blockIdx.x << lw) + (threadIdx.x & ((1 << lw) - 1));
+    const int group = threadIdx.x >> lw, groups = FP_EQ_BS >> lw;
     const double twopi = 6.283185307179586476925286766559;
     double Bs[3], Bd[3];
     if (j < A.S_out) {
@@ -93,20 +100,20 @@ __global__ void __launch_bounds__(FP_EQ_BS) fp_equilibrium_kernel(EqArgs A, int 
     for (long long i0 = (long long)blockIdx.y * G; i0 < A.n; i0 += (long long)gridDim.y * G) {
         const int gn = (int)(A.n - i0 < G ? A.n - i0 : G);
         __syncthreads();
-        if (threadIdx.x < gn) {
-            const fp_instance& in = A.inst[i0 + threadIdx.x];
+        for (int q = threadIdx.x; q < gn; q += FP_EQ_BS) {
+            const fp_instance& in = A.inst[i0 + q];
             const double d = in.d;
             const bool ok = d > 0.0 && in.flags == 0;
             const double V = 3.14159265358979323846 * d * d * d / 6.0;
             const double bT = V * A.mat.Ms / (FP_KB * A.mat.T_B);
-            double* s = si[threadIdx.x];
+            double* s = si[q];
             for (int k = 0; k < 3; ++k) s[k] = in.h_off[k];
             s[3] = ok ? bT : -1.0;
             s[4] = 1.0 / bT;
         }
         __syncthreads();
         if (j >= A.S_out) continue;
-        for (int q = 0; q < gn; ++q) {
+        for (int q = group; q < gn; q += groups) {
             const double* s = si[q];
             const size_t e = ((size_t)(i0 + q) * A.S_out + j) * 3;
             const double bT = s[3];
@@ -325,13 +332,28 @@ int fp_equilibrium(fp_ctx* ctx, const fp_instance* d_inst, int n, double* d_m, d
     A.S_out = ctx->drv.output_periods * ctx->drv.samples_per_period;
     A.m_out = d_m;
     A.dmdt_out = d_dmdt;
-    // as many instances per thread as leave eight CTAs for every SM
-    const int tiles = (A.S_out + FP_EQ_BS - 1) / FP_EQ_BS;
-    long long G = (long long)n * tiles / (8LL * ctx->num_sms);
-    G = G < 1 ? 1 : G > FP_EQ_MAXG ? FP_EQ_MAXG : G;
+    // samples a block: 128 (lw = 7), or 32 to 4 where that leaves fewer lanes without a sample.  Per
+    // instance the FP64 pipe serves about as many lanes as lanes(): whole warps with 128 to a block,
+    // whose idle warps count half beside the other blocks' (they hold their place on the SM), and
+    // with fewer some 8 more for the drive, which is formed for fewer instances per thread.  Us by
+    // 128 / by this rule / by the one thread per sample and instance before, 5,000 instances: 3
+    // samples 39 / 17 / 20, 33 70 / 49 / 81, 64 70 / 70 / 140, 129 217 / 125 / 257, 300 289 / 226 / 578, 816 632 / 617 / 1,544
+    int lw = 7;
+    auto lanes = [&](int l) {
+        const double S = A.S_out, groups = FP_EQ_BS >> l, fill = ceil(n / groups) * groups / n;
+        if (l < 7) return (ceil(S / (1 << l)) * (1 << l) + 8.0) * fill;
+        const double warps = ceil(S / 32.0) * 32.0, tiles = ceil(S / FP_EQ_BS);
+        return tiles > 1.0 ? 0.5 * (warps + tiles * FP_EQ_BS) : warps;
+    };
+    for (int l = 5; l >= FP_EQ_MINLW; --l)
+        if (lanes(l) < 0.97 * lanes(lw)) lw = l;
+    // as many instances per thread as leave eight CTAs for every SM, four or two of those without idle warps
+    const int tiles = ((A.S_out - 1) >> lw) + 1, groups = FP_EQ_BS >> lw, ctas = lw == 7 ? 8 : lw > 2 ? 4 : 2;
+    long long G = (long long)n * tiles / groups / ((long long)ctas * ctx->num_sms);
+    G = (G < 1 ? 1 : G > FP_EQ_MAXG ? FP_EQ_MAXG : G) * groups;
     const long long gy = (n + G - 1) / G;
     fp_equilibrium_kernel<<<dim3((unsigned)tiles, (unsigned)(gy < 65535 ? gy : 65535)), FP_EQ_BS, 0, (cudaStream_t)stream>>>(
-        A, (int)G);
+        A, (int)G, lw);
     if (cudaGetLastError() != cudaSuccess) return fp_fail(FP_ECUDA, "fp_equilibrium: launch failed");
     return FP_OK;
 }

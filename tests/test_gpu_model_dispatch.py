@@ -7,7 +7,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2106_08040_gb300 import build      # noqa: E402
+from paper_2106_08040_gb300 import build, workloads      # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -90,3 +90,29 @@ def test_m2_gram_at_the_lines(fp, J, N):
     Go = M.conj().T @ M
     iu = np.triu_indices(J + 1)
     assert np.abs(Gg[iu] - Go[iu]).max() <= 1e-12 * np.abs(Go).max()
+
+
+# 8 to 128 samples a block, ragged last blocks, fewer instances than groups of a block, a second round of them
+@pytest.mark.parametrize("n,S", [(1, 4), (7, 4), (33, 4), (3000, 5), (1, 64), (40, 20), (700, 33), (130, 65),
+                                 (257, 50), (3, 65), (1100, 45), (17, 816)])
+def test_equilibrium_at_the_lines(fp, n, S):
+    from oracle import models, physics, solve
+    d = workloads.DriveSpec(amp=(0.012, 0.009, 0.0), freq=(25e3, 30e3, 0.0), phase=(np.pi / 2, 0.3, 0.0),
+                            period=S / 2.5e6, samples_per_period=S, warmup_periods=1, output_periods=2)
+    inst = workloads.random_instances(n, 6, seed=S)
+    inst["d"] = np.random.default_rng(n).uniform(4e-9, 25e-9, n)
+    inst["d"][n // 2] = 0.0                                   # no moment
+    ctx = fp.Context(fp.Material(), fp.Drive(**d.__dict__), fp.Tol(), 8)
+    m = torch.full((n, 2 * S, 3), np.nan, dtype=torch.float64, device="cuda")
+    dm = torch.full_like(m, np.nan)
+    fp.fp_equilibrium(ctx, fp.instances_to_device(inst, "cuda"), n, m, dm)
+    mm, dd = m.cpu().numpy(), dm.cpu().numpy()
+    assert np.isfinite(mm).all() and np.isfinite(dd).all()
+    assert (mm[n // 2] == 0).all() and (dd[n // 2] == 0).all()
+    drv = physics.Drive(amp=d.amp, freq=d.freq, phase=d.phase, period=d.period)
+    t = solve.sample_times(drv, solve.Schedule(S, 1, 2))
+    for i in sorted(({0, 1, n // 3, n - 2, n - 1} & set(range(n))) - {n // 2}):
+        mo, do = models.equilibrium_trace(physics.Material(), drv, float(inst["d"][i]), inst["h_off"][i], t)
+        assert rel(mm[i], mo) <= 1e-13, i
+        assert rel(dd[i], do) <= 1e-12, i
+    ctx.close()

@@ -330,7 +330,7 @@ __global__ void fp_signal_kernel(const double* __restrict__ dmdt, int S_out, int
 //   X[k]        = sum_b B[k1][c][b] W_r3^(b d)                        (k1 > r1/2: conj X[S - k])
 // The FP64 pipe (2 operations a clock and SM) bounds both forms: the direct sum
 // takes 2 (k_max + 1) of them per sample, this one about r1 + 2 r2 + 2 r3, 57
-// against 1634 at S = 1632 = 17 * 12 * 8.  k1 runs fastest in both buffers, so
+// against 1634 at S = 1632 = 17 * 8 * 12.  k1 runs fastest in both buffers, so
 // neighbouring threads touch neighbouring words.  1,024 instances x 2 channels,
 // S = 1632, k_max = 816: 10.35 ms by the direct sum, about 0.45 ms here.
 struct SigPlan { int r1, r2, r3; };
@@ -414,8 +414,13 @@ static size_t sig_smem(const SigPlan& P) {
 // exceed 100 KB (two CTAs per SM; S beyond about 4,000).  Per sample: direct
 // 2 (k_max + 1); transform r1 + 2 r2 + 2 r3 scaled by the r1/2 + 1 of r1 kept
 // columns, the last stage only for the harmonics asked for, plus some 12 for
-// twiddles and indices
-static bool sig_plan(int S, int k_max, SigPlan* best) {
+// twiddles and indices.
+// A transform's CTA has a channel of few samples and stages of few threads; the direct sum a CTA
+// per instance, whose warps take the harmonics of all channels.  So short periods of several
+// channels stay with the sum (16,000 instances x 4 channels, 16 samples, 16 harmonics: 154 us, 354
+// by the transform; 48 samples, 25 harmonics 472 and 383): the times of 16,000 instances, in us,
+// fitted to 240 sizes of 4 to 180 samples on either side, decide
+static bool sig_plan(int S, int k_max, int C, SigPlan* best) {
     int div[64], nd = 0;                                  // enough for every S that fits (at most 48 divisors)
     for (int d = 1; d * d <= S && nd < 62; ++d)
         if (S % d == 0) {
@@ -433,7 +438,10 @@ static bool sig_plan(int S, int k_max, SigPlan* best) {
             const double c = 2.0 * half * r1 + 4.0 * half * r2 + 4.0 * P.r3 * (k_max + 1) / S + 12.0;
             if (c < cost && sig_smem(P) <= 100 * 1024) { cost = c; *best = P; found = true; }
         }
-    return found;
+    if (!found) return false;
+    const double transform_us = 8.0 + C * (56.0 + 0.0246 * cost * S + 0.65 * (best->r1 + best->r2 + best->r3));
+    const double direct_us = 60.0 + S * (1.8 * ((C * (k_max + 1LL) + 31) / 32) + 0.13 * C);
+    return transform_us < direct_us;
 }
 
 extern "C" int fp_signal(fp_ctx* ctx, const double* d_dmdt, int n, int k_max, const double* h_channels, int C,
@@ -454,7 +462,7 @@ extern "C" int fp_signal(fp_ctx* ctx, const double* d_dmdt, int n, int k_max, co
     // the limits are the same in every call: they belong to the process, and other host threads may launch
     SigPlan P;
     // the transform writes pairs: a result that is not 16-byte aligned takes the direct kernel
-    if ((reinterpret_cast<unsigned long long>(d_phihat) & 15ull) == 0 && sig_plan(S, k_max, &P)) {
+    if ((reinterpret_cast<unsigned long long>(d_phihat) & 15ull) == 0 && sig_plan(S, k_max, C, &P)) {
         sm = sig_smem(P);
         if (cudaFuncSetAttribute(fp_signal_fft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) != cudaSuccess)
             return fail(FP_ECUDA, "fp_signal: smem attribute");

@@ -116,3 +116,23 @@ def test_equilibrium_at_the_lines(fp, n, S):
         assert rel(mm[i], mo) <= 1e-13, i
         assert rel(dd[i], do) <= 1e-12, i
     ctx.close()
+
+
+# short periods of one and several channels, either side of the line between the transform and the direct sum
+@pytest.mark.parametrize("S,k_max,C", [(16, 15, 1), (16, 15, 4), (24, 23, 2), (36, 35, 1), (36, 18, 4), (37, 36, 2),
+                                       (37, 36, 4), (48, 24, 4), (60, 15, 1), (60, 15, 4), (64, 16, 4), (80, 20, 4)])
+def test_signal_at_the_lines(fp, S, k_max, C):
+    rng = np.random.default_rng(S + C)
+    d = workloads.DriveSpec(amp=(0.01, 0.0, 0.0), freq=(25e3,) * 3, phase=(0.0,) * 3, period=S / 2.5e6,
+                            samples_per_period=S, warmup_periods=0, output_periods=2)
+    ctx = fp.Context(fp.Material(), fp.Drive(**d.__dict__), fp.Tol(), 4)
+    n = 5
+    dm = rng.normal(size=(n, 2 * S, 3))
+    ch = rng.normal(size=(C, 3))
+    out = torch.full((n, C, k_max + 1, 2), np.nan, dtype=torch.float64, device="cuda")
+    fp.fp_signal(ctx, torch.from_numpy(dm).cuda(), n, k_max, ch, out)
+    got = out.cpu().numpy()
+    for i in range(n):
+        ref = np.fft.fft(dm[i, S:] @ ch.T, axis=0).T[:, :k_max + 1] / S
+        assert np.abs(got[i, ..., 0] + 1j * got[i, ..., 1] - ref).max() <= 1e-12 * np.abs(ref).max(), i
+    ctx.close()

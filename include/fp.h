@@ -332,7 +332,8 @@ int fp_surrogate_infer(const fp_surrogate* net, const float* d_x, int q, float* 
  * judge is the solver): d_mean [q][800] = (y_0 + y_1) / 2 and d_spread [q] =
  * ||y_0 - y_1||_2 / (2 ||mean||_2), the members' disagreement used to send a
  * query to the solver.  One last GEMM launch forms both networks' outputs side
- * by side, writes their mean and accumulates both norms per query.
+ * by side, writes their mean and accumulates both norms per query; before it,
+ * d_mean holds activations.
  * Workspace fp_surrogate_workspace_bytes(q, 2); otherwise as
  * fp_surrogate_infer. */
 int fp_surrogate_infer_ensemble(const fp_surrogate* net0, const fp_surrogate* net1, const float* d_x, int q,

@@ -936,7 +936,7 @@ const int NL[FP_SUR_LAYERS] = {FP_SUR_HIDDEN, FP_SUR_HIDDEN, FP_SUR_HIDDEN, FP_S
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct InferWs {
-    __nv_bfloat16 *x0, *h[3];      // the third buffer keeps the first network's last activations (ensemble)
+    __nv_bfloat16 *x0, *h[3];      // h[2]: the caller's output, unused until the last launch (ensemble)
     float* rowacc;                 // [q][2] (ensemble)
 };
 
@@ -949,10 +949,7 @@ size_t infer_ws(long long q, bool ensemble, unsigned char* base, InferWs* w) {
     t.h[1] = (__nv_bfloat16*)take((size_t)q * FP_SUR_HIDDEN * 2);
     t.h[2] = nullptr;
     t.rowacc = nullptr;
-    if (ensemble) {
-        t.h[2] = (__nv_bfloat16*)take((size_t)q * FP_SUR_HIDDEN * 2);
-        t.rowacc = (float*)take((size_t)q * 2 * sizeof(float));
-    }
+    if (ensemble) t.rowacc = (float*)take((size_t)q * 2 * sizeof(float));
     if (w) *w = t;
     return o;
 }
@@ -1077,7 +1074,11 @@ int fp_surrogate_infer_ensemble(const fp_surrogate* net0, const fp_surrogate* ne
     cudaStream_t st = (cudaStream_t)stream;
     if (cudaMemsetAsync(w.rowacc, 0, (size_t)q * 2 * sizeof(float), st) != cudaSuccess)
         return fp_fail(FP_ECUDA, "fp_surrogate_infer_ensemble: memset");
-    const int dst0[FP_SUR_LAYERS - 1] = {0, 1, 0, 2}, dst1[FP_SUR_LAYERS - 1] = {0, 1, 0, 1};
+    // the first network's last activations stay in h[1], the second network's in h[0]; its own way
+    // there needs a third buffer, for which the output, 3,200 bytes a query, has room until the last launch
+    static_assert(FP_SUR_HIDDEN * 2 + 255 <= FP_SUR_OUT * 4, "activations of any batch fit into its output");
+    w.h[2] = (__nv_bfloat16*)al256((size_t)d_mean);
+    const int dst0[FP_SUR_LAYERS - 1] = {0, 1, 0, 1}, dst1[FP_SUR_LAYERS - 1] = {2, 0, 2, 0};
     int rc = hidden_layers(net0, d_x, q, w, dst0, d_err, st, "fp_surrogate_infer_ensemble");
     if (rc != FP_OK) return rc;
     rc = hidden_layers(net1, d_x, q, w, dst1, d_err, st, "fp_surrogate_infer_ensemble");
@@ -1092,7 +1093,7 @@ int fp_surrogate_infer_ensemble(const fp_surrogate* net0, const fp_surrogate* ne
     P.outf = d_mean;
     P.ldf = FP_SUR_OUT;
     P.rowacc = w.rowacc;
-    const Operand op[2] = {{w.h[2], KL[4], net0->W[4], KL[4]}, {w.h[1], KL[4], net1->W[4], KL[4]}};
+    const Operand op[2] = {{w.h[1], KL[4], net0->W[4], KL[4]}, {w.h[0], KL[4], net1->W[4], KL[4]}};
     rc = gemm_out<EPI_OUT_ENSEMBLE>(op, q, NL[4], KL[4], P, st);
     if (rc != FP_OK) return fp_fail(rc, "fp_surrogate_infer_ensemble: layer 4 GEMM launch failed");
     ensemble_spread_kernel<<<(q + 255) / 256, 256, 0, st>>>(w.rowacc, q, d_spread);

@@ -1,0 +1,48 @@
+"""Surrogate calls on workspaces of the documented sizes and on outputs of any alignment."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2106_08040_gb300 import build   # noqa: E402
+from test_gpu_surrogate import random_net   # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sur():
+    build.build()
+    from paper_2106_08040_gb300 import surrogate
+    return surrogate
+
+
+def queries(n, seed):
+    return torch.from_numpy(np.random.default_rng(seed).normal(size=(n, 7)).astype(np.float32)).cuda()
+
+
+@pytest.mark.parametrize("q,offset", [(1, 0), (1, 1), (3, 7), (129, 4), (700, 0), (700, 63)])
+def test_ensemble_in_the_documented_workspace(sur, q, offset):
+    """The mean of both networks' answers: three FP32 roundings, 2^-22 of the larger answer; nothing
+    written beside the output, the spread and the workspace.  Spread: two sums of 800 squares in
+    FP32, in any order (at most 160 roundings, 1e-5), here within 1e-4."""
+    from paper_2106_08040_gb300 import _lib
+    a, b = random_net(sur, 41), random_net(sur, 42)
+    x = queries(q, 43)
+    need = sum((s + 255) // 256 * 256 for s in (128 * q, 1024 * q, 1024 * q, 8 * q))
+    ws = torch.zeros(need + 256, dtype=torch.uint8, device="cuda")
+    flat = torch.zeros(offset + q * 800 + 64, device="cuda")
+    mean, spread = flat[offset:offset + q * 800].view(q, 800), torch.zeros(q + 1, device="cuda")
+    _lib.check(_lib.lib().fp_surrogate_infer_ensemble(
+        C.byref(a.net), C.byref(b.net), C.c_void_p(x.data_ptr()), q, C.c_void_p(mean.data_ptr()),
+        C.c_void_p(spread.data_ptr()), C.c_void_p(ws.data_ptr()), C.c_ulonglong(need),
+        C.c_void_p(a._err.data_ptr()), C.c_void_p(torch.cuda.current_stream().cuda_stream)), "ensemble")
+    y0, y1 = a.infer(x), b.infer(x)
+    assert a.error_flag() == 0
+    assert bool(((mean - 0.5 * (y0 + y1)).abs() <= 2.0 ** -22 * torch.maximum(y0.abs(), y1.abs())).all())
+    ref = (y0 - y1).double().norm(dim=1) / (2 * mean.double().norm(dim=1))
+    assert float(((spread[:q] - ref).abs() / ref).max()) <= 1e-4
+    assert float(flat[:offset].abs().sum()) == 0 and float(flat[offset + q * 800:].abs().sum()) == 0
+    assert float(spread[q]) == 0 and int(ws[need:].sum()) == 0

@@ -1,0 +1,23 @@
+"""Workspace sizes of the surrogate calls (host only): what a query takes, so that a caller's
+buffer of this size stays large enough.  Each array is rounded up to 256 bytes.
+"""
+import pytest
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2106_08040_gb300 import build
+    build.build()
+    from paper_2106_08040_gb300 import _lib
+    return _lib.lib()
+
+
+def total(*sizes):
+    return sum((s + 255) // 256 * 256 for s in sizes)
+
+
+@pytest.mark.parametrize("q", [1, 7, 257, 4096, 1024000])
+def test_inference_and_ensemble(lib, q):
+    x0, h = 128 * q, 1024 * q                        # bf16 inputs (64 wide) and activations (512 wide)
+    assert lib.fp_surrogate_workspace_bytes(q, 0) <= total(x0, h, h)
+    assert lib.fp_surrogate_workspace_bytes(q, 2) <= total(x0, h, h, 8 * q)

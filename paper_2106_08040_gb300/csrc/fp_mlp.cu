@@ -960,7 +960,8 @@ struct TrainWs {
     __nv_bfloat16* h[FP_SUR_LAYERS - 1];                  // [q][512] activations (inputs of layers 1..4)
     __nv_bfloat16* hT[FP_SUR_LAYERS - 1];                 // [512][ldt]
     __nv_bfloat16 *g4, *g4T;                              // [q][800], [800][ldt]
-    __nv_bfloat16* g[2];                                  // [q][512] ping-pong
+    __nv_bfloat16* g[2];                                  // [q][512] ping-pong, in h[0] and h[1]: after the forward
+                                                          // pass their transposes alone are read
     __nv_bfloat16* gT[FP_SUR_LAYERS - 1];                 // [512][ldt]: G^T of layers 0..3, kept for the dW launch
     int ldt;
 };
@@ -979,7 +980,7 @@ size_t train_ws(long long q, unsigned char* base, TrainWs* w) {
     }
     t.g4 = (__nv_bfloat16*)take((size_t)q * FP_SUR_OUT * 2);
     t.g4T = (__nv_bfloat16*)take((size_t)FP_SUR_OUT * t.ldt * 2);
-    for (int i = 0; i < 2; ++i) t.g[i] = (__nv_bfloat16*)take((size_t)q * FP_SUR_HIDDEN * 2);
+    for (int i = 0; i < 2; ++i) t.g[i] = t.h[i];
     for (int l = 0; l < FP_SUR_LAYERS - 1; ++l) t.gT[l] = (__nv_bfloat16*)take((size_t)FP_SUR_HIDDEN * t.ldt * 2);
     if (w) *w = t;
     return o;

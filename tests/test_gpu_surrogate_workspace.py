@@ -46,3 +46,29 @@ def test_ensemble_in_the_documented_workspace(sur, q, offset):
     assert float(((spread[:q] - ref).abs() / ref).max()) <= 1e-4
     assert float(flat[:offset].abs().sum()) == 0 and float(flat[offset + q * 800:].abs().sum()) == 0
     assert float(spread[q]) == 0 and int(ws[need:].sum()) == 0
+
+
+@pytest.mark.parametrize("q", [8, 264, 4096])
+def test_gradients_in_the_documented_workspace(sur, q):
+    """Gradients in a workspace of garbage against those in a fresh one: sums over the batch in one
+    order, so the same bits; the loss is added up by atomics."""
+    from paper_2106_08040_gb300 import _lib
+    s = random_net(sur, 51)
+    x = queries(q, 52)
+    y = torch.from_numpy(np.random.default_rng(53).normal(size=(q, 800)).astype(np.float32)).cuda()
+    need = sum((b + 255) // 256 * 256 for b in [128 * q] * 2 + [2048 * q, 1024 * q, 1024 * q] * 4 + [1600 * q] * 2 +
+               [1024 * q] * 4)
+    ws = torch.full((need + 256,), 0xC1, dtype=torch.uint8, device="cuda")
+    s.grad(x, y)
+    ref = [g.clone() for g in s.gW + s.gb]
+    loss = float(s._loss.item())
+    for g in s.gW + s.gb:
+        g.fill_(float("nan"))
+    _lib.check(_lib.lib().fp_surrogate_grad(
+        C.byref(s.train_state), C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), q, C.c_void_p(s._loss.data_ptr()),
+        s._gW, s._gb, C.c_void_p(ws.data_ptr()), C.c_ulonglong(need), C.c_void_p(s._err.data_ptr()),
+        C.c_void_p(torch.cuda.current_stream().cuda_stream)), "grad")
+    assert s.error_flag() == 0
+    assert all(torch.equal(a, b) for a, b in zip(s.gW + s.gb, ref))
+    assert abs(float(s._loss.item()) - loss) <= 1e-5 * loss
+    assert bool((ws[need:] == 0xC1).all())

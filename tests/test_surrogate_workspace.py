@@ -21,3 +21,12 @@ def test_inference_and_ensemble(lib, q):
     x0, h = 128 * q, 1024 * q                        # bf16 inputs (64 wide) and activations (512 wide)
     assert lib.fp_surrogate_workspace_bytes(q, 0) <= total(x0, h, h)
     assert lib.fp_surrogate_workspace_bytes(q, 2) <= total(x0, h, h, 8 * q)
+
+
+@pytest.mark.parametrize("q", [8, 64, 4096, 65536])
+def test_training(lib, q):
+    """bf16 inputs and their transpose; per hidden layer FP32 pre-activations, activations and their
+    transpose; output cotangents and their transpose; two pairs of hidden cotangents."""
+    layer = [2048 * q, 1024 * q, 1024 * q]
+    assert lib.fp_surrogate_workspace_bytes(q, 1) <= total(128 * q, 128 * q, *layer * 4, 1600 * q, 1600 * q,
+                                                           *[1024 * q] * 4)

@@ -13,6 +13,7 @@ fp_surrogate_grad / fp_surrogate_adam; every arithmetic step of inference and
 training runs in those kernels.
 """
 import ctypes as C
+import functools
 
 import numpy as np
 
@@ -33,6 +34,20 @@ def _stream(stream):
     import torch
     s = stream if stream is not None else torch.cuda.current_stream()
     return C.c_void_p(s.cuda_stream)
+
+
+@functools.lru_cache(maxsize=256)
+def _workspace_bytes(q, training):
+    nb = int(_lib.lib().fp_surrogate_workspace_bytes(int(q), int(training)))
+    if nb < 0:
+        check(nb, "fp_surrogate_workspace_bytes")
+    return nb
+
+
+class _Workspace:
+    def __init__(self, tensor):
+        self.tensor, self.size = tensor, tensor.numel()
+        self.ptr, self.bytes = C.c_void_p(tensor.data_ptr()), C.c_ulonglong(self.size)
 
 
 def features(inst):
@@ -79,7 +94,8 @@ class Surrogate:
         self.out_shift = torch.zeros(N_OUT, **f32)
         self.out_scale = torch.ones(N_OUT, **f32)
         self.step = 0
-        self._ws = {}
+        self._ws = {}                     # workspaces by stream
+        self._captured = {}               # those that a captured graph may write to
         self._err = torch.zeros(1, dtype=torch.int32, device=self.device)
         self._loss = torch.zeros(1, **f32)
         self._build_structs()
@@ -131,15 +147,31 @@ class Surrogate:
             ys = np.full(y.shape[1], max(float(np.sqrt(np.mean((y - mu) ** 2))), 1e-30))
         self.out_scale.copy_(torch.from_numpy(ys.astype(np.float32)))
 
-    def workspace(self, q, training):
+    def workspace(self, q, training, stream=None):
+        """Device workspace for one call of q queries on `stream` (the current one by default), as
+        long as fp_surrogate_workspace_bytes says.  The calls on a stream run one after another, so they
+        share one buffer, which grows to the largest of them; each stream has its own.  A buffer
+        that a capture has seen is kept as long as this object, since a replay writes to it;
+        graphs captured from one stream share it and must not replay at the same time."""
+        return self._buffer(q, training, stream)[0].tensor[:_workspace_bytes(q, training)]
+
+    def _buffer(self, q, training, stream):
+        """The workspace of a call and the handle of its stream."""
         import torch
-        key = (q, training)
-        if key not in self._ws:
-            nb = _lib.lib().fp_surrogate_workspace_bytes(int(q), int(training))
-            if nb < 0:
-                check(int(nb), "fp_surrogate_workspace_bytes")
-            self._ws[key] = torch.empty(int(nb), dtype=torch.uint8, device=self.device)
-        return self._ws[key]
+        s = stream if stream is not None else torch.cuda.current_stream()
+        nb = _workspace_bytes(q, training)
+        ws = self._ws.get(s.cuda_stream)
+        if ws is None or ws.size < nb:
+            with torch.cuda.stream(s):
+                # the one that this replaces goes back to the allocator in the order of its stream
+                ws = self._ws[s.cuda_stream] = _Workspace(torch.empty(nb, dtype=torch.uint8, device=self.device))
+        capturing = torch.cuda.is_current_stream_capturing()
+        if stream is not None and not capturing:
+            with torch.cuda.stream(s):
+                capturing = torch.cuda.is_current_stream_capturing()
+        if capturing:
+            self._captured[ws.tensor.data_ptr()] = ws.tensor
+        return ws, C.c_void_p(s.cuda_stream)
 
     # ----------------------------------------------------------- inference --
     def infer(self, x, out=None, stream=None):
@@ -147,19 +179,18 @@ class Surrogate:
         import torch
         q = x.shape[0]
         y = out if out is not None else torch.empty((q, N_OUT), dtype=torch.float32, device=self.device)
-        ws = self.workspace(q, 0)
-        check(_lib.lib().fp_surrogate_infer(C.byref(self.net), _p(x), int(q), _p(y), _p(ws), C.c_ulonglong(ws.numel()),
-                                            _p(self._err), _stream(stream)), "fp_surrogate_infer")
+        ws, st = self._buffer(q, 0, stream)
+        check(_lib.lib().fp_surrogate_infer(C.byref(self.net), _p(x), int(q), _p(y), ws.ptr, ws.bytes,
+                                            _p(self._err), st), "fp_surrogate_infer")
         return y
 
     # ------------------------------------------------------------ training --
     def grad(self, x, y, stream=None):
         """Loss (sum of squared normalised errors) into self._loss, gradients into self.gW/gb."""
         q = x.shape[0]
-        ws = self.workspace(q, 1)
+        ws, st = self._buffer(q, 1, stream)
         check(_lib.lib().fp_surrogate_grad(C.byref(self.train_state), _p(x), _p(y), int(q), _p(self._loss),
-                                           self._gW, self._gb, _p(ws), C.c_ulonglong(ws.numel()), _p(self._err),
-                                           _stream(stream)), "fp_surrogate_grad")
+                                           self._gW, self._gb, ws.ptr, ws.bytes, _p(self._err), st), "fp_surrogate_grad")
         return self._loss
 
     def adam(self, lr, beta1=0.9, beta2=0.999, eps=1e-8, stream=None):

@@ -75,13 +75,11 @@ class Ensemble:
         q = x.shape[0]
         mean = torch.empty((q, surrogate.N_OUT), dtype=torch.float32, device=a.device)
         spread = torch.empty((q,), dtype=torch.float32, device=a.device)
-        ws = a.workspace(q, 2)
-        s = stream if stream is not None else torch.cuda.current_stream()
+        ws, st = a._buffer(q, 2, stream)
         _lib.check(_lib.lib().fp_surrogate_infer_ensemble(C.byref(a.net), C.byref(b.net), C.c_void_p(x.data_ptr()),
                                                           int(q), C.c_void_p(mean.data_ptr()),
-                                                          C.c_void_p(spread.data_ptr()), C.c_void_p(ws.data_ptr()),
-                                                          C.c_ulonglong(ws.numel()), C.c_void_p(a._err.data_ptr()),
-                                                          C.c_void_p(s.cuda_stream)), "fp_surrogate_infer_ensemble")
+                                                          C.c_void_p(spread.data_ptr()), ws.ptr, ws.bytes,
+                                                          C.c_void_p(a._err.data_ptr()), st), "fp_surrogate_infer_ensemble")
         return mean, spread
 
     def save(self, path, **meta):

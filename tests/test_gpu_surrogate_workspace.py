@@ -72,3 +72,37 @@ def test_gradients_in_the_documented_workspace(sur, q):
     assert all(torch.equal(a, b) for a, b in zip(s.gW + s.gb, ref))
     assert abs(float(s._loss.item()) - loss) <= 1e-5 * loss
     assert bool((ws[need:] == 0xC1).all())
+
+
+def test_two_streams_at_one_batch_size(sur):
+    """Inference, ensemble and gradients on two streams side by side repeat what they give alone."""
+    from paper_2106_08040_gb300 import surrogate_train
+    nets = [random_net(sur, 61), random_net(sur, 62)]
+    ens = surrogate_train.Ensemble(nets)
+    q = 3000
+    xs = [queries(q, 63), queries(q, 64)]
+    alone = [(nets[0].infer(x), ens.infer(x)[0]) for x in xs]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    outs = [[], []]
+    for i in range(30):
+        for k, s in enumerate(streams):
+            with torch.cuda.stream(s):
+                outs[k].append(nets[0].infer(xs[k], stream=s) if i % 2 else ens.infer(xs[k], stream=s)[0])
+    torch.cuda.synchronize()
+    for k in range(2):
+        for i, o in enumerate(outs[k]):
+            assert torch.equal(o, alone[k][0] if i % 2 else alone[k][1]), (k, i)
+    assert nets[0].error_flag() == 0
+
+
+def test_memory_does_not_grow_with_the_batch_sizes(sur):
+    s = random_net(sur, 65)
+    x = queries(5000, 66)
+    y = torch.empty((5000, 800), device="cuda")
+    s.infer(x, out=y)
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    for q in range(1000, 5000, 40):
+        s.infer(x[:q], out=y[:q])
+    assert torch.cuda.memory_allocated() == before

@@ -731,7 +731,9 @@ int launch_t(const Maps<EPI>& maps, const EpiParams& P, int ntiles, cudaStream_t
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, mlp_gemm_kernel<BN, EPI>, maps, P, ntiles) == cudaSuccess ? FP_OK : FP_ECUDA;
+    if (cudaLaunchKernelEx(&cfg, mlp_gemm_kernel<BN, EPI>, maps, P, ntiles) == cudaSuccess) return FP_OK;
+    cudaGetLastError();                                    // reported here: not left for the next call's check
+    return FP_ECUDA;
 }
 
 int vec_of(const void* p, int ld, int size) {

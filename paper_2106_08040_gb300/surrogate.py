@@ -162,9 +162,13 @@ class Surrogate:
         nb = _workspace_bytes(q, training)
         ws = self._ws.get(s.cuda_stream)
         if ws is None or ws.size < nb:
-            with torch.cuda.stream(s):
-                # the one that this replaces goes back to the allocator in the order of its stream
-                ws = self._ws[s.cuda_stream] = _Workspace(torch.empty(nb, dtype=torch.uint8, device=self.device))
+            if stream is None:
+                ws = _Workspace(torch.empty(nb, dtype=torch.uint8, device=self.device))
+            else:
+                with torch.cuda.stream(s):
+                    ws = _Workspace(torch.empty(nb, dtype=torch.uint8, device=self.device))
+            # the one that this replaces goes back to the allocator in the order of its stream
+            self._ws[s.cuda_stream] = ws
         capturing = torch.cuda.is_current_stream_capturing()
         if stream is not None and not capturing:
             with torch.cuda.stream(s):

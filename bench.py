@@ -400,7 +400,7 @@ def models_leg(fp, dev, peak64, Q=96, J2=96):
     1024 voxels, and the M1 fit of a Q-element dictionary (8 diameters x 12
     anisotropies at one angle, synthetic phi_hat of the solver's shape) against
     one measured matrix.  fp_m1_fit reads the dictionary twice (filter, then
-    row errors): HBM-bound."""
+    row errors): bound by the FP64 pipe."""
     import torch
     from paper_2106_08040_gb300 import workloads
     dspec, inst = workloads.system_matrix_workload()
@@ -438,9 +438,10 @@ def models_leg(fp, dev, peak64, Q=96, J2=96):
     ms_m1 = e[2].elapsed_time(e[3]) / reps
     by = 2.0 * (phi.numel() + Sm.numel()) * 8 + (a.numel() + eps.numel()) * 8
     hbm, src = measured_peak("hbm_gbs", 6800.0)
-    # FP64 work per (element, dictionary entry): S conj(Phi) (8), |Phi|^2 (4) and
-    # |S|^2 (3) in the first pass; a Phi (6), S - a Phi (2), |r|^2 (4) in the second
-    fl = 27.0 * Q * n * C * K1
+    # FP64 work per (element, dictionary entry): S conj(Phi) (8) and |Phi|^2 (4) in the
+    # first pass (|S|^2 is formed once for all elements); S - a Phi (8) and |r|^2 (4) in
+    # the second
+    fl = 24.0 * Q * n * C * K1
     out = {"m0_voxels": n, "m0_ms": ms_m0, "m0_voxel_periods_per_s": n * 2 / (ms_m0 * 1e-3),
            "m1_dictionary": Q, "m1_ms": ms_m1, "m1_fits_per_s": Q / (ms_m1 * 1e-3),
            "m1_roofline": {"bound": "alu", "achieved": fl / (ms_m1 * 1e-3) / 1e12, "peak": peak64, "unit": "TFLOP/s",
@@ -472,15 +473,15 @@ def models_leg(fp, dev, peak64, Q=96, J2=96):
     w, obj, res, sv, srank = fp.fp_m2_solve(G.cpu().numpy(), J2, 21)
     t_host = time.time() - t0
     rows = A2 * N2 * C * len(ks)
-    tiles = -(-(J2 + 1) // 16)
-    flops = 8.0 * rows * (16 * 16) * tiles * (tiles + 1) / 2      # complex multiply-adds of the computed tiles
+    nt = -(-(J2 + 1) // 4)                                        # 4 x 4 register tiles, u <= v
+    flops = 8.0 * rows * 16 * nt * (nt + 1) / 2                   # complex multiply-adds of the computed tiles
     flops_alg = 8.0 * rows * (J2 + 1) * (J2 + 2) / 2              # upper triangle of the Gram matrix
     out.update({"m2_gram_ms": ms_g, "m2_rows": rows, "m2_J": J2, "m2_angles": A2, "m2_voxels": N2,
                 "m2_host_solve_s": t_host, "m2_rank": srank, "m2_nonzero_weights": int((w > 1e-12 * w.max()).sum()),
                 "m2_gram_roofline": {"bound": "alu", "achieved": flops_alg / (ms_g * 1e-3) / 1e12, "peak": peak64,
                                      "unit": "TFLOP/s", "frac": flops_alg / (ms_g * 1e-3) / 1e12 / peak64,
                                      "executed_over_algorithmic": flops / flops_alg,
-                                     "kernel": "fp_m2_gram_kernel (FP64, upper-triangle tiles)"}})
+                                     "kernel": "fp_m2_gram_micro_kernel (FP64, 4 x 4 register tiles of the upper triangle)"}})
     del phi2, a2, S2
     return out
 

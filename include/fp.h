@@ -145,7 +145,13 @@ int fp_num_samples(const fp_ctx* ctx);
  * or non-positive K < 0, d <= 0 get FP_STATUS_BAD_INPUT and zero outputs.
  * The launch uses the context's factor scratch and work counter (allocated
  * by fp_setup): calls on one context must not overlap in time (issue them on
- * one stream, or give each stream its own context). */
+ * one stream, or give each stream its own context).  With 5 stages a batch of
+ * at most one instance per SM keeps its factors in shared memory, one CTA to
+ * an SM, a larger one in the scratch, two CTAs to an SM; the results are the
+ * same bits.  The choice is made from n alone, so two such batches on two
+ * streams share no SM: two of 152 instances of degree 16 take 167 ms side by
+ * side, 166 ms with the layout of the larger ones, but one alone 104 ms
+ * instead of 150. */
 int fp_solve_batch(fp_ctx* ctx, const fp_instance* d_inst, int n,
                    double* d_m, double* d_dmdt, int* d_status, int* d_stats,
                    void* stream);
@@ -317,7 +323,8 @@ typedef struct {
 
 /* Device workspace (bytes) for q queries: inference (training = 0), one
  * gradient evaluation (training = 1; q must then be a multiple of 8), or
- * ensemble inference (training = 2, fp_surrogate_infer_ensemble). */
+ * ensemble inference (training = 2, fp_surrogate_infer_ensemble).  2,176,
+ * 23,936 and 2,184 bytes a query, each array rounded up to 256 bytes. */
 long long fp_surrogate_workspace_bytes(int q, int training);
 
 /* Surrogate inference: d_x [q][7] f32 -> d_y [q][800] f32.  d_err (device

@@ -8,7 +8,7 @@
 // epilogues, which also store transposed copies (X^T, G^T) and by keeping W^T
 // beside W, so one kernel shape serves forward, dX and dW.
 //
-// Tile: 128 rows (UMMA M = 128), BN columns (64..256), K blocks of 64 bf16 =
+// Tile: 128 rows (UMMA M = 128), BN columns (32..256), K blocks of 64 bf16 =
 // one 128-byte swizzle row; one persistent CTA per SM walks its tiles through
 // an STAGES-deep TMA ring.  Warp 0 lane 0 issues TMA, warp 1 lane 0 issues
 // tcgen05.mma into a ring of TMEM accumulators (warp 1 owns the allocation),
@@ -17,13 +17,15 @@
 // Every wait is bounded in time; a wait that gives up sets *err and the CTA
 // drains its copies and MMAs and frees TMEM before it returns.
 //
-// What bounds it (GB300, 262,144 queries): the 512 -> 512 layers take 136 us and read 11 TB/s of
-// operands from L2, which is its limit, at 48 KB per 128 x 256 x 64 block; the first layer (K = 64)
-// 105 us, its epilogue; both output layers together 0.55 ms, again 11 TB/s.  1,024,000 queries
-// through two networks: 13.7 -> 6.36 ms.  Small batches are a chain of launches: 257 queries
-// 88 -> 32 us with narrow tiles and overlapped launches; a training step of 4096 queries
-// 594 -> 191 us with one launch for all weight gradients, one for the bias gradients and one for
-// the optimiser (25 kernels before, 13 now).
+// What bounds it (GB300, 262,144 queries): no unit of the chip, by its counters.  A 512 -> 512 layer takes
+// 136 us with the tensor pipe busy 42 % of the time, L2 at 40 % of its sector rate (52 % of its tag rate; it
+// delivers 10.7 TB/s, 48 KB per 128 x 256 x 64 block) and HBM at 44 %; both output layers together take
+// 561 us with 32, 38 (45) and 30 %.  What is left is the chain of one CTA per SM: the loads in
+// flight, the MMAs behind them and the epilogue's turn with the accumulators.  The first
+// layer (K = 64) takes 105 us, its epilogue.  1,024,000 queries through two networks: 13.7 -> 6.32 ms.
+// Small batches are a chain of launches: 257 queries 88 -> 32 us with narrow tiles and overlapped
+// launches; a training step of 4096 queries 594 -> 192 us with one launch for all weight
+// gradients, one for the bias gradients and one for the optimiser (25 kernels before, 13 now).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -771,7 +773,11 @@ int gemm_bn(const Operand* op, int M, int N, int K, EpiParams P, cudaStream_t st
 // tiles' columns (epilogue and operand reads; the 48 stand for the A rows and the fill of the
 // pipeline), so large batches take the widest tile, and a few hundred queries, which are
 // latency-bound, a narrow one with a short epilogue (257 queries: 24 tiles of 64 columns in
-// one wave).  The K order, and with it the result, is the same for all.
+// one wave).  The K order, and with it the result, is the same for all.  One inference by hidden
+// tiles of 64 / 128 / 256 columns: 28.8 / 32.5 / 39.6 us at 257 queries, 32.4 / 35.9 / 43.2 at 2,432
+// and 41.6 / 35.4 / 43.1 at 2,433, 49.9 / 42.6 / 51.5 at 4,800, 74 / 59 / 54 at 8,500; by output tiles of 32 /
+// 80 / 160: 28.7 / 29.8 / 30.9 at 257, 31.8 / 29.8 / 30.9 at 1,200, 42.6 / 38.5 / 36.0 at 3,000.  Over 32 sizes up to
+// 90,000 queries the rule is within 3 % of the best, but 9 % at 19,457 to 22,000 (112 us; 103 by 256).
 long long tile_cost(int M, int N, int BN) {
     const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN), sms = num_sms();
     return (tiles + sms - 1) / sms * (BN + 48);

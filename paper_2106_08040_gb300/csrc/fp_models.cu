@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(FP_EQ_BS) fp_equilibrium_kernel(EqArgs A, int 
 // and SM), HBM runs at a quarter of its rate: so max |S|^2 is formed by the
 // first element's CTAs alone, and the residual's two products and subtraction
 // are two fused operations a component.  96 elements x 1,024 voxels x 1,634
-// columns with fp_nrmse: 5.41 ms -> 3.40 ms; the FP64 floor is 3.07 ms.
+// columns with fp_nrmse: 5.41 ms -> 3.37 ms; the FP64 floor is 3.07 ms.
 // pass 1: a = sum S conj(Phi) / sum |Phi|^2 and (q = 0) max |S| per column
 template <int COLS, int VG>
 __global__ void __launch_bounds__(COLS * VG) fp_m1_pass1(const double2* __restrict__ phi, const double2* __restrict__ S, int N, int CK,

@@ -313,8 +313,8 @@ def phi_hat(params, h_off, fpctx, L, k_max, channels):
     """Differentiable phi_hat (torch.autograd) of the batched solve: params
     [n, 4] = (K, d, theta, phi), h_off [n, 3]; the backward pass is fp_grad
     (discrete adjoint).  Raises if any instance of either pass does not
-    converge.  At L = 16 the adjoint needs a 3-stage context (a 5-stage one
-    exceeds the shared memory of a CTA)."""
+    converge.  At L = 16 some instances do not with 5 stages (their segment
+    replay stalls): use a 3-stage context there."""
     global _PHIHAT
     if _PHIHAT is None:
         _PHIHAT = _autograd_function()
